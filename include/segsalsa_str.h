@@ -264,8 +264,8 @@ int segsalsa_str_linear_solve_static(const float* rhs, float* z, int32_t H, int3
  * device time in milliseconds since the last reset. Kernel kinds (index):
  *   0 fused sweep (prox + dual + rhs partials), 1 row FFT forward (with partial gather),
  *   2 column solve, 3 row FFT inverse, 4 diagnostics (residual / objective), 5 other,
- *   6 MLR class model (set_spectra), 7 reverse-pass kernels (backward), 8 z-update fused
- *   over a thread-block cluster (replaces 1-3 where the tiling selects it).
+ *   6 MLR class model (set_spectra), 7 reverse-pass kernels (backward), 8 z-update in one
+ *   launch (pixel domain, cluster or tickets; replaces 1-3).
  * launches and ms point to arrays of at least 9 entries (host memory). kernel_stats works
  * with profiling off too; then ms is not filled. reset_stats zeroes both. */
 int segsalsa_str_set_profiling(segsalsa_str_t* h, int32_t on);
@@ -307,7 +307,12 @@ int segsalsa_str_traffic_model(const segsalsa_str_t* h, double* sweep_bytes,
  *                 tiling; column segments are lengthened where the column pass would need
  *                 more than 512 threads; one-unit row form only; measured slower than the
  *                 three launches chained by programmatic dependent launch: 145x145, K = 16,
- *                 36.3 vs 30.8 us per iteration); 0 = the library's choice (three launches).
+ *                 36.3 vs 30.8 us per iteration); 0 = the library's choice: in FP32, with
+                 row_pipe = 0 and weights whose squared sum is at most 1 (the Gaussian ones),
+                 one launch in the pixel domain (no transforms: the other fields but tile_rows
+                 are then unused), else three launches. get_tiling reports zfuse = 1 and
+                 row_pipe = 0 for a handle that leaves this choice to the library, and a
+                 complete tiling with those two values leaves it too.
  *                 A fused request that the band or the device cannot hold runs three
  *                 launches (get_tiling reports 1).
  *   row_pipe    : form of the two row-transform passes: 1 = one CTA per (row, class block);

@@ -367,6 +367,7 @@ struct RowArgs {
   // source of rhs: dense [n][K] (src != null) or the sweep partials
   const T* src;
   const T* P;            // [tiles][EHmax][EWmax][K]
+  int pstr, pquad, ptile;  // strides of P as the sweep wrote it (gather_rhs only; see SweepArgs)
   int ntx, EHmax, EWmax;
   const int* covY;       // [H][2]: (tile row << 16 | ext row), -1 when absent
   const int* covX;       // [W][2]: (tile col << 16 | ext col)
@@ -395,7 +396,7 @@ __device__ __forceinline__ T gather_rhs(const RowArgs<T>& a, int y, int x, int k
       if (cx < 0) continue;
       const int tx = cx >> 16, ex = cx & 0xffff;
       const size_t t = (size_t)ty * a.ntx + tx;
-      v += a.P[((t * a.EHmax + ey) * a.EWmax + ex) * a.K + k];
+      v += a.P[t * a.ptile + (size_t)(ey * a.EWmax + ex) * a.pstr + (size_t)(k >> 2) * a.pquad + (k & 3)];
     }
   }
   return v;

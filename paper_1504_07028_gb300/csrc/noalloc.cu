@@ -23,6 +23,7 @@
 
 #include "../../include/segsalsa_str.h"
 #include "fft.cuh"
+#include "zlocal.cuh"
 
 namespace sgs {
 namespace {
@@ -148,6 +149,21 @@ extern "C" int segsalsa_str_linear_solve_static(const float* rhs, float* z, int3
   const size_t col_smem = (size_t)H * CB * sizeof(float2);
   if (col_smem > 200 * 1024) return SEGSALSA_ERR_OOM;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  if (c_omega <= ZL_MAX_C) {
+    // the pixel-domain form needs no scratch and no tables
+    ZlArgs za{};
+    za.H = H; za.W = W; za.K = K; za.src = rhs; za.z = z;
+    za.q = zl_coef(c_omega);
+    // this thread's last geometry keeps its work split
+    static thread_local int lH = 0, lW = 0, lK = 0;
+    static thread_local ZlPlan lp;
+    if (lH != H || lW != W || lK != K) {
+      lp = zl_plan(H, W, K);
+      lH = H; lW = W; lK = K;
+    }
+    za.p = lp;
+    return launch_zlocal(za, st) == cudaSuccess ? SEGSALSA_OK : SEGSALSA_ERR_CUDA;
+  }
 
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) return SEGSALSA_ERR_CUDA;

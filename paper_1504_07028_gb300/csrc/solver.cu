@@ -24,6 +24,7 @@
 #include "aux.cuh"
 #include "fft.cuh"
 #include "zfused.cuh"
+#include "zlocal.cuh"
 #include "launch.h"
 #include "mlr.cuh"
 #include "adjoint.cuh"
@@ -153,6 +154,11 @@ struct Plan {
   // (ordered tickets; the one-unit row form only)
   int zs, zs_threads, zs_grid;
   size_t zs_smem;
+  // z-update in the pixel domain (FP32, the library's own choice of z-update; used while the
+  // weights' squared sum allows it, see zlocal.cuh)
+  int zl;
+  ZlPlan zlp;
+  size_t pslot;            // values of the rhs partials (class quads padded where zl)
   int nproj_blk, nprior_blk;
   // wide patches (M >= 3): two-launch sweep (gram + transpose tiles) writing a dense rhs
   int wide, wntx1, wntiles1, wnblk2;
@@ -395,6 +401,15 @@ static int make_plan(const segsalsa_str_params* pr, Plan& pl, std::string& msg,
       if (pl.zs_smem > 227 * 1024) pl.zs = 0;
     }
   }
+  // the library's own choice of z-update in FP32: the pixel-domain one. Fields that select a
+  // form of the row transforms turn it off; a complete tiling with zfuse = 1 and row_pipe = 0
+  // is what get_tiling reports for such a handle.
+  {
+    const bool own = !tl || (tl->row_pipe == 0 && (tl->zfuse == 0 || (tl->zfuse == 1 && tl->tile_rows && tl->row_pairs && tl->col_block && tl->row_threads && tl->col_rows)));
+    pl.zl = sizeof(T) == 4 && own;
+    if (pl.zl) pl.zlp = zl_plan(H, W, K);
+    pl.pslot = (size_t)pl.ntiles * pl.EHmax * pl.EWmax * (pl.zl ? (K + 3) / 4 * 4 : K);
+  }
   // diagnostics
   // one pixel per thread (projection) and tiles of PRIOR_TH x PRIOR_TW pixels (prior): one
   // round per block up to eight blocks per SM, grid-stride rounds beyond (small images need
@@ -434,6 +449,7 @@ struct Buffers {
   unsigned int* zctr;  // [4] work-ticket counters of the one-launch z-update (0 between launches)
   T* omega;
   int *covY, *covX, *offX;
+  int* offYq;  // [H][2] row offsets of the rhs partials in class quads (pixel-domain z-update)
   T *beta, *gain, *wfac;
   int* nwarm;
   cplx<T>*tw, *chirp, *bhat;
@@ -450,7 +466,7 @@ static size_t carve(const Plan& pl, char* base, Buffers<T>& b) {
   b.dcmp = c.take<T>((size_t)pl.n * (pl.K + 2) + 64 / sizeof(T));
   b.d2 = c.take<T>(2 * (size_t)pl.L * nK + 64 / sizeof(T));
   const size_t tslot = (size_t)pl.ntiles * pl.EHmax * pl.EWmax * pl.K;
-  b.P = c.take<T>(tslot);
+  b.P = c.take<T>(pl.pslot);
   b.P2 = c.take<T>(tslot);
   b.zp = c.take<T>(nK);
   b.tmp = c.take<T>(nK);
@@ -470,6 +486,7 @@ static size_t carve(const Plan& pl, char* base, Buffers<T>& b) {
   b.covY = c.take<int>((size_t)pl.H * MAXCOV);
   b.covX = c.take<int>((size_t)pl.W * MAXCOV);
   b.offX = c.take<int>((size_t)pl.W * MAXCOV);
+  b.offYq = pl.zl ? c.take<int>((size_t)pl.H * MAXCOV) : nullptr;
   b.beta = c.take<T>(pl.Wh);
   b.gain = c.take<T>(pl.Wh);
   b.wfac = c.take<T>(pl.Wh);
@@ -505,10 +522,14 @@ class Solver : public SolverBase {
   // the local duals are held in compact form (b.dcmp, written by the affine fused sweep)
   // rather than in full form (b.dloc: set_probs, set_state, the simplex and wide sweeps)
   bool dl_cmp = false;
+  bool p_quads = false;    // layout of the last sweep's rhs partials (see p_strides)
 
   // The form of the local duals the handle's sweeps keep from iteration to iteration (graphs
   // are captured in it): compact for the affine fused sweep, full otherwise.
-  bool dl_steady() const { return pl.wide || (g4 == SEGSALSA_G4_SIMPLEX ? !dl_cmp : dl_cmp); }
+  // The rhs partials likewise: the layout that the z-update in use reads.
+  bool dl_steady() const {
+    return pl.wide || ((g4 == SEGSALSA_G4_SIMPLEX ? !dl_cmp : dl_cmp) && p_quads == zl_now());
+  }
   int64_t nlaunch[NKIND] = {0};
   double ms[NKIND] = {0};
   bool profiling = false;
@@ -623,6 +644,16 @@ class Solver : public SolverBase {
       }
       SGS_CUDA(cudaMemcpyAsync(b.offX, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice, st));
       SGS_CUDA(cudaStreamSynchronize(st));  // `off` leaves scope
+      if (pl.zl) {
+        off.assign(pl.covY.size(), -1);
+        for (size_t i = 0; i < off.size(); ++i) {
+          const int cy = pl.covY[i];
+          if (cy >= 0)
+            off[i] = ((cy >> 16) * pl.ntx * ((pl.K + 3) / 4) * pl.EHmax + (cy & 0xffff)) * pl.EWmax;
+        }
+        SGS_CUDA(cudaMemcpyAsync(b.offYq, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice, st));
+        SGS_CUDA(cudaStreamSynchronize(st));
+      }
     }
     // column solve coefficients, per kx: (a + 2c) - c (S + S^-1) = (c/beta)(1 - beta S)(1 - beta/S)
     std::vector<T> beta(Wh), gain(Wh), wfac(Wh);
@@ -723,6 +754,26 @@ class Solver : public SolverBase {
     return a;
   }
 
+  // Dense rhs [n][K] from the sweep's partials.
+  int gather_dense(T* dst) {
+    const size_t nK = (size_t)pl.n * pl.K;
+    RowArgs<T> ra = row_args(nullptr, dst);
+    p_strides(p_quads, ra.pstr, ra.pquad, ra.ptile);
+    SGS_LAUNCH(KIND_OTHER, (k_gather_dense<T><<<grid1(nK), AUX_THREADS, 0, st>>>(ra)));
+    return SEGSALSA_OK;
+  }
+  // Strides of the rhs partials: planes of four classes for the pixel-domain z-update, else
+  // pixel-major.
+  void p_strides(bool quads, int& str, int& quad, int& tile) const {
+    const int px = pl.EHmax * pl.EWmax;
+    str = quads ? 4 : pl.K;
+    quad = quads ? 4 * px : 4;
+    tile = px * (quads ? (pl.K + 3) / 4 * 4 : pl.K);
+  }
+
+  // Whether the z-update runs in the pixel domain (the weights may change it: set_weights).
+  bool zl_now() const { return pl.zl && c_omega <= ZL_MAX_C; }
+
   // Bring the full form up to date (d1 = c1 p, d4 = c4 1) and make it the one in use.
   int dl_to_full() {
     if (!dl_cmp) return SEGSALSA_OK;
@@ -737,6 +788,25 @@ class Solver : public SolverBase {
   // partials, or the dense rhs of the wide-patch sweep)
   int z_update(const T* src, T* zout) {
     if (!src && pl.wide) src = b.rhsd;
+    if constexpr (sizeof(T) == 4) {
+      if (zl_now()) {
+        if (!src && !p_quads) {  // partials of a sweep before the weights changed
+          if (int rc = gather_dense(b.rhsd)) return rc;
+          src = b.rhsd;
+        }
+        ZlArgs za{};
+        za.H = pl.H; za.W = pl.W; za.K = pl.K; za.p = pl.zlp;
+        za.src = src; za.P = b.P; za.ntx = pl.ntx; za.EHmax = pl.EHmax; za.EWmax = pl.EWmax;
+        za.offY = b.offYq; za.covX = b.covX; za.z = zout;
+        za.q = zl_coef(c_omega);
+        SGS_CUDA(launch(KIND_ZF, [&]() { return launch_zlocal(za, st); }));
+        return SEGSALSA_OK;
+      }
+    }
+    if (!src && p_quads) {
+      if (int rc = gather_dense(b.rhsd)) return rc;
+      src = b.rhsd;
+    }
     const RowArgs<T> ra = row_args(src, zout);
     if (pl.zf_cs) {
       ZfArgs<T> za{};
@@ -819,6 +889,8 @@ class Solver : public SolverBase {
     a.EHmax = pl.EHmax; a.EWmax = pl.EWmax;
     a.z = b.z; a.p = b.p; a.dloc = b.dloc; a.d2 = b.d2; a.P = b.P; a.P2 = b.P2;
     a.dcmp = b.dcmp;
+    p_quads = zl_now();
+    p_strides(p_quads, a.pstr, a.pquad, a.ptile);
     a.cin = (!simplex && dl_cmp) ? 1 : 0;
     a.diag_sq = b.dsq; a.omega = b.omega;
     a.tau = (T)(lambda / mu); a.mu = (T)mu; a.invK = (T)(1.0 / pl.K); a.sp = sp;
@@ -1146,8 +1218,7 @@ class Solver : public SolverBase {
       if (rhs_dense || pl.wide) {
         if ((rc = copy_out(rhs, b.rhsd, nK, dev))) return rc;
       } else {
-        const RowArgs<T> ra = row_args(nullptr, b.tmp);
-        SGS_LAUNCH(KIND_OTHER, (k_gather_dense<T><<<grid1(nK), AUX_THREADS, 0, st>>>(ra)));
+        if ((rc = gather_dense(b.tmp))) return rc;
         if ((rc = copy_out(rhs, b.tmp, nK, dev))) return rc;
       }
     }
@@ -1243,7 +1314,7 @@ class Solver : public SolverBase {
     t.tile_rows = pl.THmax; t.row_pairs = pl.QB; t.col_block = pl.CB;
     t.row_threads = pl.row_threads; t.col_rows = pl.col_rows;
     t.zfuse = pl.zs ? 3 : pl.zf_cs ? pl.zf_cs : 1;
-    t.row_pipe = pl.p2 ? 3 : pl.rp ? 2 : 1;
+    t.row_pipe = pl.zl ? 0 : pl.p2 ? 3 : pl.rp ? 2 : 1;
     return t;
   }
 
@@ -1269,7 +1340,7 @@ class Solver : public SolverBase {
   }
   void advance(int len) override {
     iter += len;
-    if (pl.zs || pl.zf_cs) {
+    if (pl.zs || pl.zf_cs || zl_now()) {
       nlaunch[KIND_ZF] += len;
     } else {
       nlaunch[KIND_ROWF] += len; nlaunch[KIND_COL] += len; nlaunch[KIND_ROWI] += len;
@@ -1376,7 +1447,7 @@ class Solver : public SolverBase {
     if (pl.wide) return fail(SEGSALSA_ERR_ARG, "the reverse pass covers patches up to 5 x 5 (M <= 2)");
     const int K = pl.K, L = pl.L, n = pl.n;
     const size_t nK = (size_t)n * K, nloc = 3 * nK, n2 = 2 * (size_t)L * nK;
-    const size_t tslot = (size_t)pl.ntiles * pl.EHmax * pl.EWmax * K;
+    const size_t tslot = pl.pslot;
     const size_t st_elems = nK + nloc + n2 + tslot;          // z, d1/d3/d4, d2, rhs partials
     const int nseg = (iters + every - 1) / every;
     const int blocks = (n + ADJ_THREADS / pl.G - 1) / (ADJ_THREADS / pl.G);
@@ -1946,7 +2017,9 @@ struct segsalsa_str_batch {
           const int rc = pr.precision == SEGSALSA_FP32 ? sgs::make_plan<float>(&pr, pl, msg, &t)
                                                        : sgs::make_plan<double>(&pr, pl, msg, &t);
           if (rc) return false;
-          key.push_back(pl.THmax); key.push_back(pl.QB); key.push_back(pl.CB);
+          key.push_back(pl.THmax); key.push_back(pl.zl);
+          if (pl.zl) continue;                  // no row or column pass to tile
+          key.push_back(pl.QB); key.push_back(pl.CB);
           key.push_back(pl.row.threads); key.push_back(pl.NSEG); key.push_back(pl.zf_cs);
           key.push_back(pl.rp);
           key.push_back(pl.p2);

@@ -39,8 +39,11 @@ struct SweepArgs {
   int cin;               // affine g4: the local duals come in compact form (else full form);
                          // the affine sweep writes the compact form, the simplex sweep the full
   T* d2;                 // [n][L][K][2]
-  T* P;                  // [tiles][EHmax][EWmax][K]  partial sums of G^T(u + d)
-  T* P2;                 // DIAG: partial sums of G^T d (dual residual)
+  T* P;                  // per tile: partial sums of G^T(u + d) over [EHmax][EWmax] pixels; class k of
+                         // pixel q at q * pstr + (k / 4) * pquad + k % 4 of the tile's ptile values
+  int pstr, pquad, ptile;  // K, 4, EHmax EWmax K: pixel-major; 4, 4 EHmax EWmax, ...: planes of
+                           // four classes (the z-update of zlocal.cuh reads whole quads)
+  T* P2;                 // DIAG: partial sums of G^T d (dual residual), [tiles][EHmax][EWmax][K]
   double* diag_sq;       // DIAG: per tile sum of squared dual changes (primal residual)
   const T* omega;        // [L] shift weights
   T tau;                 // lambda / mu
@@ -155,12 +158,14 @@ __device__ __forceinline__ void issue_row(const SweepArgs<T>& a, size_t pix0, in
 // to exclusive slots (columns c .. c+E-1 of the tile+halo row), the block synchronises, and
 // the owner of each (column, class) sums the E slots in order s = 0..E-1 and stores the result
 // straight into row `ey` of the tile's partials (each tile+halo row is flushed exactly once).
-// Slots of idle columns stay zero; the caller synchronises before the slots are reused.
+// Slots of idle columns stay zero; the caller synchronises before the slots are reused. Pt / Pt2
+// already point at this thread's class.
 template <typename T, int G, int E, bool DIAG>
 __device__ __forceinline__ void flush_row(const T (&w)[E], const T (&w2)[DIAG ? E : 1], bool colok,
                                           int c, int g, T* slots, T* slots2, T* Pt, T* Pt2,
-                                          int ey, int EWmax, int EW, int K) {
-  constexpr int SW = 256 / G + E - 1;
+                                          int ey, int EWmax, int EW, int K, int pstr) {
+  constexpr int NCT = 256 / G;
+  constexpr int SW = NCT + E - 1;
   if (colok) {
 #pragma unroll
     for (int s = 0; s < E; ++s) {
@@ -169,18 +174,21 @@ __device__ __forceinline__ void flush_row(const T (&w)[E], const T (&w2)[DIAG ? 
     }
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < EW * G; e += blockDim.x) {
-    const int col = e / G, lane = e & (G - 1);
-    if (lane >= K) continue;
-    T sum = T(0), sum2 = T(0);
+  if (g >= K) return;
+  const int q = ey * EWmax;
 #pragma unroll
-    for (int s = 0; s < E; ++s) {
-      sum += slots[(s * SW + col) * G + lane];
-      if constexpr (DIAG) sum2 += slots2[(s * SW + col) * G + lane];
+  for (int r = 0; r < (SW + NCT - 1) / NCT; ++r) {
+    const int col = c + r * NCT;
+    if (col < EW) {
+      T sum = T(0), sum2 = T(0);
+#pragma unroll
+      for (int s = 0; s < E; ++s) {
+        sum += slots[(s * SW + col) * G + g];
+        if constexpr (DIAG) sum2 += slots2[(s * SW + col) * G + g];
+      }
+      Pt[(q + col) * pstr] = sum;
+      if constexpr (DIAG) Pt2[(size_t)(q + col) * K] = sum2;
     }
-    const size_t o = ((size_t)ey * EWmax + col) * K + lane;
-    Pt[o] = sum;
-    if constexpr (DIAG) Pt2[o] = sum2;
   }
 }
 
@@ -224,8 +232,10 @@ __global__ void __launch_bounds__(256, sweep_min_blocks<T, M, DIAG>()) k_sweep(c
   const int EH = TH + 2 * M + 1, EW = TW + 2 * M + 1;
   const int K = KEQ ? G : a.K;
   (void)EH;
-  T* Pt = a.P + (size_t)tile * a.EHmax * a.EWmax * K;   // this tile's partials (tile + halo)
-  T* Pt2 = DIAG ? a.P2 + (size_t)tile * a.EHmax * a.EWmax * K : nullptr;
+  // this tile's partials (tile + halo), at the thread's class
+  const int gl = threadIdx.x % G;
+  T* Pt = a.P + (size_t)tile * a.ptile + (gl >> 2) * a.pquad + (gl & 3);
+  T* Pt2 = DIAG ? a.P2 + (size_t)tile * a.EHmax * a.EWmax * K + gl : nullptr;
 
   if (threadIdx.x == 0) {
     mbar_init(&mbar[0], 1);
@@ -465,7 +475,7 @@ __global__ void __launch_bounds__(256, sweep_min_blocks<T, M, DIAG>()) k_sweep(c
     }
     // ---- flush the finished top window row (tile+halo row r), in a fixed summation order
     flush_row<T, G, E, DIAG>(accW[0], accW2[0], colok, c, g, slots, slots2, Pt, Pt2, r, EWs,
-                             EW, K);
+                             EW, K, a.pstr);
 #pragma unroll
     for (int rr = 0; rr < E - 1; ++rr)
 #pragma unroll
@@ -487,7 +497,7 @@ __global__ void __launch_bounds__(256, sweep_min_blocks<T, M, DIAG>()) k_sweep(c
   for (int rr = 0; rr < E - 1; ++rr) {
     __syncthreads();  // the previous flush's owners are done with the slots
     flush_row<T, G, E, DIAG>(accW[rr], accW2[DIAG ? rr : 0], colok, c, g, slots, slots2, Pt, Pt2,
-                             TH + rr, EWs, EW, K);
+                             TH + rr, EWs, EW, K, a.pstr);
   }
   if constexpr (DIAG) {
     const double t = block_sum_w<T>(sq, red32);
