@@ -106,21 +106,30 @@ __device__ __forceinline__ void pdl_trigger() {
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 }
 
-// Launch with the programmatic-serialization attribute (see pdl_wait).
+// Launch with the programmatic-serialization attribute (see pdl_wait). max_shared: ask for the
+// largest shared-memory carve-out. An SM changes its carve-out only when it is idle, so the CTAs of
+// a dependent kernel with another one wait for the SM's last CTA of its predecessor.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                              cudaStream_t st, Args&&... args) {
+inline cudaError_t launch_pdl_carve(bool max_shared, void (*kern)(KArgs...), dim3 grid, dim3 block,
+                                    size_t smem, cudaStream_t st, Args&&... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  at[1].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = max_shared ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                              cudaStream_t st, Args&&... args) {
+  return launch_pdl_carve(false, kern, grid, block, smem, st, static_cast<Args&&>(args)...);
 }
 
 // Identity of the calling thread's current CUDA context: unique for the life of the process, so

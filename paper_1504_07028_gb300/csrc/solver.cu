@@ -133,7 +133,8 @@ static std::vector<double> make_weights(const segsalsa_str_params* pr) {
 struct Plan {
   int H, W, K, M, L, n, G, NC;
   int ntx, nty, THmax, EHmax, EWmax, ntiles;
-  size_t sweep_smem, sweep_smem_diag;
+  int sweep_nt;                                    // threads of a sweep CTA: 256 or 64
+  size_t sweep_smem[2][2], sweep_smem_simplex[2];  // [local duals in compact form][traced], [traced]
   int Wh, Mf, blue, QB, nqblk;
   RowLaunch row;
   // pipelined row passes (persistent CTAs): on/off, vertical-cover stage slots, shared memory
@@ -211,25 +212,36 @@ static int make_plan(const segsalsa_str_params* pr, Plan& pl, std::string& msg,
   pl.n = pl.H * pl.W;
   const int K = pl.K, M = pl.M, H = pl.H, W = pl.W;
   pl.G = K <= 4 ? 4 : K <= 8 ? 8 : K <= 16 ? 16 : 32;
-  // columns per tile: 256/G, fewer when a CTA's shared memory (two row stages, the z tile and
-  // the accumulators) would not fit
+  // columns per tile: threads / G, fewer when a CTA's shared memory (two row stages, the z tile
+  // and the accumulators) would not fit; tile height: the largest of {16, 12, 8, 6, 4} that still
+  // gives two CTAs per SM (152 SMs). With more than one tile row every tile must be at least
+  // 2M+1 rows high
   const int cand[] = {16, 12, 8, 6, 4};
-  for (pl.NC = 256 / pl.G; pl.NC > 1; --pl.NC) {
-    const size_t s = sweep_smem_bytes<T>(pl.NC, 16 + 2 * M + 1, pl.NC + 2 * M + 1, pl.G, pl.L, K, true);
-    if (s <= 220 * 1024) break;
-  }
-  pl.ntx = (W + pl.NC - 1) / pl.NC;
-  // tile height: the largest of {16, 12, 8, 6, 4} that still gives two CTAs per SM (152 SMs);
-  // with more than one tile row every tile must be at least 2M+1 rows high
-  pl.THmax = 0;
-  int fallback = 0;
-  for (int th : cand) {
-    const int nty = (H + th - 1) / th;
-    if (nty > 1 && H / nty < 2 * M + 1) continue;
-    fallback = th;
-    if ((long long)nty * pl.ntx >= 304) { pl.THmax = th; break; }
-  }
-  if (!pl.THmax) pl.THmax = fallback ? fallback : H;
+  auto smem_of = [&](int nt, int nc, int eh, bool diag, bool compact, bool simplex) {
+    return sweep_smem_bytes<T>(nt, nc, eh, nc + 2 * M + 1, pl.G, pl.L, K, diag, compact, simplex);
+  };
+  auto tiles_of = [&](int nt) {
+    pl.sweep_nt = nt;
+    for (pl.NC = nt / pl.G; pl.NC > 1; --pl.NC)
+      if (smem_of(nt, pl.NC, 16 + 2 * M + 1, true, false, false) <= 220 * 1024) break;
+    pl.ntx = (W + pl.NC - 1) / pl.NC;
+    pl.THmax = 0;
+    int fallback = 0;
+    for (int th : cand) {
+      const int nty = (H + th - 1) / th;
+      if (nty > 1 && H / nty < 2 * M + 1) continue;
+      fallback = th;
+      if ((long long)nty * pl.ntx >= 304) { pl.THmax = th; break; }
+    }
+    if (!pl.THmax) pl.THmax = fallback ? fallback : H;
+    return (long long)((H + pl.THmax - 1) / pl.THmax) * pl.ntx;
+  };
+  // images that leave SMs without a tile of 256 threads at any height: CTAs of 64 threads, four
+  // times as many tiles (64 x 64, K = 4: 16 -> 64 CTAs, FP64 sweep 103 -> 46 us; CTAs of 32 threads
+  // gained nothing over that, and 97 x 509 with its 200 tiles takes 18.5 us per iteration with 256
+  // threads, 28.1 with 64)
+  if (tiles_of(256) < 152 && pl.NC == 256 / pl.G && sweep_small_ok(M, pl.G) && W >= 2 * (64 / pl.G))
+    tiles_of(64);
   if (tl && tl->tile_rows) {
     // requested height, raised until every tile of a multi-row tiling has >= 2M+1 rows
     int th = tl->tile_rows;
@@ -239,8 +251,13 @@ static int make_plan(const segsalsa_str_params* pr, Plan& pl, std::string& msg,
   pl.nty = (H + pl.THmax - 1) / pl.THmax;
   pl.EHmax = pl.THmax + 2 * M + 1;
   pl.EWmax = pl.NC + 2 * M + 1;
-  pl.sweep_smem = sweep_smem_bytes<T>(pl.NC, pl.EHmax, pl.EWmax, pl.G, pl.L, K, false);
-  pl.sweep_smem_diag = sweep_smem_bytes<T>(pl.NC, pl.EHmax, pl.EWmax, pl.G, pl.L, K, true);
+  size_t most = 0;
+  for (int d = 0; d < 2; ++d) {
+    for (int c = 0; c < 2; ++c)
+      most = std::max(most, pl.sweep_smem[c][d] = smem_of(pl.sweep_nt, pl.NC, pl.EHmax, d, c, false));
+    pl.sweep_smem_simplex[d] = smem_of(pl.sweep_nt, pl.NC, pl.EHmax, d, false, true);
+    most = std::max(most, pl.sweep_smem_simplex[d]);
+  }
   pl.wide = M >= 3;
   pl.wntx1 = (W + 256 / pl.G - 1) / (256 / pl.G);
   pl.wntiles1 = pl.wntx1 * ((H + WG_TH - 1) / WG_TH);
@@ -250,7 +267,7 @@ static int make_plan(const segsalsa_str_params* pr, Plan& pl, std::string& msg,
     if (wide_gram_smem<T>(M, pl.G) > 227 * 1024) {
       msg = "wide-patch tiles do not fit in shared memory"; return SEGSALSA_ERR_ARG;
     }
-  } else if (pl.sweep_smem_diag > 227 * 1024) {
+  } else if (most > 227 * 1024) {
     msg = "tile does not fit in shared memory"; return SEGSALSA_ERR_ARG;
   }
   pl.ntiles = pl.ntx * pl.nty;
@@ -589,8 +606,10 @@ class Solver : public SolverBase {
     if (pr->stream) st = reinterpret_cast<cudaStream_t>(pr->stream);
     else { SGS_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking)); own_stream = true; }
     if (pl.wide) SGS_CUDA(prepare_wide<T>(pl.M, pl.G));
-    else if (pl.K == pl.G && pl.NC == 256 / pl.G) SGS_CUDA(prepare_sweep_keq<T>(pl.M, pl.G, pl.sweep_smem, pl.sweep_smem_diag));
-    else SGS_CUDA(prepare_sweep<T>(pl.M, pl.G, pl.sweep_smem, pl.sweep_smem_diag));
+    else {
+      const SweepArgs<T> none{};
+      for (int d = 0; d < 2; ++d) SGS_CUDA(sweep_launch(none, false, d, 0, pl.sweep_smem[0][d]));
+    }
     SGS_CUDA(prepare_fft<T>(pl.row, pl.col_smem));
     if (pl.zf_cs && zfused_max_clusters<T>(pl.zf_cs, pl.zf_threads, pl.zf_smem) < 1) pl.zf_cs = 0;
     if (pl.zs) {
@@ -862,6 +881,13 @@ class Solver : public SolverBase {
     return SEGSALSA_OK;
   }
 
+  cudaError_t sweep_launch(const SweepArgs<T>& a, bool simplex, bool diag, int tiles, size_t smem) {
+    const int nt = pl.sweep_nt;
+    if (simplex) return launch_sweep_simplex<T>(a, pl.M, pl.G, nt, diag, tiles, smem, st);
+    if (pl.K == pl.G && pl.NC == nt / pl.G) return launch_sweep_keq<T>(a, pl.M, pl.G, nt, diag, tiles, smem, st);
+    return launch_sweep<T>(a, pl.M, pl.G, nt, diag, tiles, smem, st);
+  }
+
   int sweep(bool diag) {
     int rc;
     if (pl.wide) {
@@ -897,12 +923,9 @@ class Solver : public SolverBase {
     a.err = b.err;
     a.budget = wait_budget;
     a.probe = wait_probe ? 16u : 0u;
-    const size_t smem = diag ? pl.sweep_smem_diag : pl.sweep_smem;
-    SGS_CUDA(launch(KIND_SWEEP, [&]() {
-      if (simplex) return launch_sweep_simplex<T>(a, pl.M, pl.G, diag, pl.ntiles, smem, st);
-      return pl.K == pl.G && pl.NC == 256 / pl.G ? launch_sweep_keq<T>(a, pl.M, pl.G, diag, pl.ntiles, smem, st)
-                          : launch_sweep<T>(a, pl.M, pl.G, diag, pl.ntiles, smem, st);
-    }));
+    a.mu4 = (T)(4.0 / mu);
+    const size_t smem = simplex ? pl.sweep_smem_simplex[diag] : pl.sweep_smem[a.cin][diag];
+    SGS_CUDA(launch(KIND_SWEEP, [&]() { return sweep_launch(a, simplex, diag, pl.ntiles, smem); }));
     if (!simplex) dl_cmp = true;
     return SEGSALSA_OK;
   }
@@ -1382,7 +1405,7 @@ class Solver : public SolverBase {
     if (mode != SEGSALSA_G4_AFFINE && mode != SEGSALSA_G4_SIMPLEX) return fail(SEGSALSA_ERR_ARG, "bad g4 mode");
     if (mode == g4) return SEGSALSA_OK;
     if (mode == SEGSALSA_G4_SIMPLEX && !pl.wide)  // the wide kernels are prepared at create
-      SGS_CUDA(prepare_sweep_simplex<T>(pl.M, pl.G, pl.sweep_smem, pl.sweep_smem_diag));
+      for (int d = 0; d < 2; ++d) SGS_CUDA(sweep_launch(SweepArgs<T>{}, true, d, 0, pl.sweep_smem_simplex[d]));
     SGS_CUDA(cudaStreamSynchronize(st));
     for (auto& kv : chunks)
       if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);

@@ -4,15 +4,9 @@
 
 namespace sgs {
 template <typename T>
-cudaError_t launch_sweep_keq(const SweepArgs<T>& a, int M, int G, bool diag, int tiles,
-                             size_t smem, cudaStream_t st) {
-  return launch_sweep_variant<T, false, true>(a, M, G, diag, tiles, smem, st);
+cudaError_t launch_sweep_keq(const SweepArgs<T>& a, int M, int G, int nt, bool diag, int tiles, size_t smem,
+                             cudaStream_t st) {
+  return launch_sweep_variant<T, false, true>(a, M, G, nt, diag, tiles, smem, st);
 }
-template <typename T>
-cudaError_t prepare_sweep_keq(int M, int G, size_t smem, size_t smem_diag) {
-  return prepare_sweep_variant<T, false, true>(M, G, smem, smem_diag);
-}
-template cudaError_t prepare_sweep_keq<float>(int, int, size_t, size_t);
-template cudaError_t launch_sweep_keq<float>(const SweepArgs<float>&, int, int, bool, int, size_t,
-                                         cudaStream_t);
+template cudaError_t launch_sweep_keq<float>(const SweepArgs<float>&, int, int, int, bool, int, size_t, cudaStream_t);
 }  // namespace sgs
