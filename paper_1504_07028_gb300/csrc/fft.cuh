@@ -156,6 +156,29 @@ __device__ __forceinline__ int qdiv(int t, uint32_t mg) {
   return mg ? (int)__umulhi((uint32_t)t, mg) : t;
 }
 
+// v[r] *= w^r, r < R, from w and w^4 (the latter used for R > 5).
+template <int R, typename C>
+__device__ __forceinline__ void twiddle_powers(C* v, const C w1, const C w4t) {
+  v[1] = cmul(v[1], w1);
+  if constexpr (R > 2) {
+    const C w2 = cmul(w1, w1);
+    v[2] = cmul(v[2], w2);
+    if constexpr (R > 3) {
+      const C w3 = cmul(w2, w1);
+      v[3] = cmul(v[3], w3);
+      if constexpr (R > 4) {
+        const C w4 = (R > 5) ? w4t : cmul(w2, w2);
+        v[4] = cmul(v[4], w4);
+        if constexpr (R > 5) {
+          v[5] = cmul(v[5], cmul(w4, w1));
+          v[6] = cmul(v[6], cmul(w4, w2));
+        }
+        if constexpr (R > 7) v[7] = cmul(v[7], cmul(w4, w3));
+      }
+    }
+  }
+}
+
 // One forward Stockham stage of radix R in {2,3,4,5,7,8} on B = 2^lgB interleaved sequences
 // X[n * B + b], out of place: each work item is one radix-R butterfly reading Xin and writing
 // Xout; the caller synchronises the block between stages.
@@ -174,27 +197,15 @@ __device__ __forceinline__ void fft_stage(const cplx<T>* __restrict__ Xin, cplx<
     C v[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = Xin[px<T>((t + r * nb) * S + b)];
-    // twiddles w^r, w = tw[j * stride]: w and (for R > 5) w^4 from the table, the other
-    // powers by at most two products
-    {
-      const C w1 = tw[j * stride];
-      v[1] = cmul(v[1], w1);
-      if (R > 2) {
-        const C w2 = cmul(w1, w1);
-        v[2] = cmul(v[2], w2);
-        if (R > 3) {
-          const C w3 = cmul(w2, w1);
-          v[3] = cmul(v[3], w3);
-          if (R > 4) {
-            const C w4 = (R > 5) ? tw[4 * j * stride] : cmul(w2, w2);
-            v[4] = cmul(v[4], w4);
-            if (R > 5) {
-              v[5] = cmul(v[5], cmul(w4, w1));
-              v[6] = cmul(v[6], cmul(w4, w2));
-            }
-            if (R > 7) v[7] = cmul(v[7], cmul(w4, w3));
-          }
-        }
+    // twiddles w^r, w = tw[j * stride], none in the first stage (Ns = 1). FP32: w and (for R > 5)
+    // w^4 from the table, the other powers by at most two products; FP64, whose products are scarce:
+    // every power from the table (r j stride < Mf)
+    if (Ns > 1) {
+      if constexpr (sizeof(T) == 8) {
+#pragma unroll
+        for (int r = 1; r < R; ++r) v[r] = cmul(v[r], tw[r * j * stride]);
+      } else {
+        twiddle_powers<R>(v, tw[j * stride], R > 5 ? tw[4 * j * stride] : C{});
       }
     }
     Dft<R, C>::run(v);
@@ -1279,23 +1290,12 @@ __device__ __forceinline__ void p2_twdft(int it, cplx<T> (&v)[R], const cplx<T>*
   constexpr int STRIDE = NB / NS;
   const int t = it / B;
   const int j = t - (t / NS) * NS;
-  if constexpr (NS > 1) {
-    const C w1 = tw[j * STRIDE];
-    v[1] = cmul(v[1], w1);
-    if constexpr (R > 2) {
-      const C w2 = cmul(w1, w1);
-      v[2] = cmul(v[2], w2);
-      if constexpr (R > 3) {
-        const C w3 = cmul(w2, w1);
-        v[3] = cmul(v[3], w3);
-        if constexpr (R > 4) {
-          const C w4 = tw[4 * j * STRIDE];
-          v[4] = cmul(v[4], w4);
-          v[5] = cmul(v[5], cmul(w4, w1));
-          v[6] = cmul(v[6], cmul(w4, w2));
-          v[7] = cmul(v[7], cmul(w4, w3));
-        }
-      }
+  if constexpr (NS > 1) {   // as fft_stage
+    if constexpr (sizeof(T) == 8) {
+#pragma unroll
+      for (int r = 1; r < R; ++r) v[r] = cmul(v[r], tw[r * j * STRIDE]);
+    } else {
+      twiddle_powers<R>(v, tw[j * STRIDE], R > 5 ? tw[4 * j * STRIDE] : C{});
     }
   }
   Dft<R, C>::run(v);
