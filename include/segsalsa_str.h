@@ -177,7 +177,8 @@ int segsalsa_str_set_weights(segsalsa_str_t* h, const double* weights);
  * backwards, recomputing each segment's states from its checkpoint: the adjoint of the z-update
  * is the z-update itself (G^T G is symmetric), the adjoints of the MPOs of g1..g4 are their
  * Jacobians applied per pixel, and the adjoint of J is J^T. Device memory for the checkpoints
- * and one segment's states is allocated for the call and released before it returns. The
+ * and one segment's states is allocated for the call and released before it returns, except that
+ * the handle keeps it for its next call, until destroy, while it is at most 64 MiB. The
  * handle ends at iteration `iters`, as after set_probs + solve(iters).
  * Covers Schatten p = 1, 2 and infinity, g4 on the affine set or on the probability simplex
  * (set_g4), and patches up to 5x5 (M <= 2); SEGSALSA_ERR_ARG for wider patches. The

@@ -24,61 +24,60 @@
 
 namespace sgs {
 
-// Value and four tangents (d/da, d/db, d/dc, d/dtau). Kept in a namespace of its own: its
-// sqrt / fmax are found by argument-dependent lookup and hide nothing for plain numbers.
+// Value and one tangent: lane g of a pixel's group carries d/da, d/db, d/dc or d/dtau (g mod 4), the
+// value being the same in all. (With all four tangents in every lane, five quotients in the data
+// prox and 5 additions a parameter in the warp sums the kernel took 822 FP64 operations a pixel and
+// class, 709 us at 256 x 256, K = 8; it is bound by the FP64 unit's two lanes a clock. Now 530 us; FP32
+// 57 -> 44 us, bound by issue slots.) Kept in a namespace of its own: its sqrt /
+// fmax are found by argument-dependent lookup and hide nothing for plain numbers.
 namespace dual {
 template <typename T>
-struct Dual4 {
+struct Dual {
   T v;
-  T d[4];
-  __device__ Dual4() : v(T(0)) { d[0] = d[1] = d[2] = d[3] = T(0); }
-  __device__ Dual4(double x) : v(T(x)) { d[0] = d[1] = d[2] = d[3] = T(0); }
+  T d;
+  __device__ Dual() : v(T(0)), d(T(0)) {}
+  __device__ Dual(double x) : v(T(x)), d(T(0)) {}
 };
-template <typename T> __device__ __forceinline__ Dual4<T> operator+(Dual4<T> x, Dual4<T> y) {
-  Dual4<T> r; r.v = x.v + y.v;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) r.d[i] = x.d[i] + y.d[i];
+template <typename T> __device__ __forceinline__ Dual<T> operator+(Dual<T> x, Dual<T> y) {
+  Dual<T> r; r.v = x.v + y.v;
+  r.d = x.d + y.d;
   return r;
 }
-template <typename T> __device__ __forceinline__ Dual4<T> operator-(Dual4<T> x, Dual4<T> y) {
-  Dual4<T> r; r.v = x.v - y.v;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) r.d[i] = x.d[i] - y.d[i];
+template <typename T> __device__ __forceinline__ Dual<T> operator-(Dual<T> x, Dual<T> y) {
+  Dual<T> r; r.v = x.v - y.v;
+  r.d = x.d - y.d;
   return r;
 }
-template <typename T> __device__ __forceinline__ Dual4<T> operator-(Dual4<T> x) {
-  Dual4<T> r; r.v = -x.v;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) r.d[i] = -x.d[i];
+template <typename T> __device__ __forceinline__ Dual<T> operator-(Dual<T> x) {
+  Dual<T> r; r.v = -x.v;
+  r.d = -x.d;
   return r;
 }
-template <typename T> __device__ __forceinline__ Dual4<T> operator*(Dual4<T> x, Dual4<T> y) {
-  Dual4<T> r; r.v = x.v * y.v;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) r.d[i] = x.d[i] * y.v + x.v * y.d[i];
+template <typename T> __device__ __forceinline__ Dual<T> operator*(Dual<T> x, Dual<T> y) {
+  Dual<T> r; r.v = x.v * y.v;
+  r.d = x.d * y.v + x.v * y.d;
   return r;
 }
-template <typename T> __device__ __forceinline__ Dual4<T> operator/(Dual4<T> x, Dual4<T> y) {
-  Dual4<T> r; r.v = x.v / y.v;
-  const T iy = T(1) / y.v;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) r.d[i] = (x.d[i] - r.v * y.d[i]) * iy;
+// One reciprocal serves the value (with a Newton correction of the quotient) and the tangent.
+template <typename T> __device__ __forceinline__ Dual<T> operator/(Dual<T> x, Dual<T> y) {
+  const T iy = T(1) / y.v, q = x.v * iy;
+  Dual<T> r; r.v = fma(fma(-q, y.v, x.v), iy, q);
+  r.d = (x.d - r.v * y.d) * iy;
   return r;
 }
-template <typename T> __device__ __forceinline__ bool operator>(Dual4<T> x, Dual4<T> y) { return x.v > y.v; }
-template <typename T> __device__ __forceinline__ bool operator>=(Dual4<T> x, Dual4<T> y) { return x.v >= y.v; }
-template <typename T> __device__ __forceinline__ Dual4<T> sqrt(Dual4<T> x) {
-  Dual4<T> r; r.v = ::sqrt(x.v);
+template <typename T> __device__ __forceinline__ bool operator>(Dual<T> x, Dual<T> y) { return x.v > y.v; }
+template <typename T> __device__ __forceinline__ bool operator>=(Dual<T> x, Dual<T> y) { return x.v >= y.v; }
+template <typename T> __device__ __forceinline__ Dual<T> sqrt(Dual<T> x) {
+  Dual<T> r; r.v = ::sqrt(x.v);
   const T h = r.v > T(0) ? T(0.5) / r.v : T(0);   // a clamped zero carries no tangent
-#pragma unroll
-  for (int i = 0; i < 4; ++i) r.d[i] = x.d[i] * h;
+  r.d = x.d * h;
   return r;
 }
-template <typename T> __device__ __forceinline__ Dual4<T> fmax(Dual4<T> x, Dual4<T> y) {
+template <typename T> __device__ __forceinline__ Dual<T> fmax(Dual<T> x, Dual<T> y) {
   return x.v >= y.v ? x : y;
 }
 }  // namespace dual
-using dual::Dual4;
+using dual::Dual;
 
 struct AdjShape {
   int H, W, K, n;
@@ -102,6 +101,7 @@ struct AdjArgs {
   double* part;       // block partials [NP][blocks]: tau, omega_0..omega_{L-1}, S (= <D bbar, D z^{k+1}>)
   const T* omega;
   T tau, mu, invK;
+  T mu4;              // 4 / mu
   int sp;
   int simplex;        // g4 on the probability simplex (else on the affine set 1^T xi = 1)
 };
@@ -173,20 +173,22 @@ __global__ void __launch_bounds__(ADJ_THREADS, 2) k_adj_vjp(const AdjArgs<T> a) 
     vv[j] = w * (zw[dy + 1][dx] - zw[dy][dx]) - dv;
   }
   const T pv = group_sum<G>(pk * v1), pp = group_sum<G>(pk * pk);
-  const T qq = T(4) * pp / a.mu;
+  const T qq = a.mu4 * pp;
   const T disc = sqrt(pv * pv + qq);
   const T t = (pv >= T(0)) ? T(0.5) * (pv + disc) : (T(0.5) * qq) / (disc - pv);
+  const T imt = T(1) / (a.mu * t), idisc = T(1) / disc;   // the pixel's two reciprocals
   T ga = T(0), gb = T(0), gc = T(0);
 #pragma unroll
   for (int j = 0; j < L; ++j) { ga += vh[j] * vh[j]; gb += vh[j] * vv[j]; gc += vv[j] * vv[j]; }
   ga = group_sum<G>(ga); gb = group_sum<G>(gb); gc = group_sum<G>(gc);
-  Dual4<T> Da(0.0), Db(0.0), Dc(0.0), Dt(0.0);
-  Da.v = ga; Da.d[0] = T(1);
-  Db.v = gb; Db.d[1] = T(1);
-  Dc.v = gc; Dc.d[2] = T(1);
-  Dt.v = a.tau; Dt.d[3] = T(1);
-  Dual4<T> A11, A12, A22;
-  schatten_coeffs<Dual4<T>>(Da, Db, Dc, Dt, a.sp, A11, A12, A22);
+  Dual<T> Da(0.0), Db(0.0), Dc(0.0), Dt(0.0);
+  const int tan = g & 3;
+  Da.v = ga; Da.d = tan == 0 ? T(1) : T(0);
+  Db.v = gb; Db.d = tan == 1 ? T(1) : T(0);
+  Dc.v = gc; Dc.d = tan == 2 ? T(1) : T(0);
+  Dt.v = a.tau; Dt.d = tan == 3 ? T(1) : T(0);
+  Dual<T> A11, A12, A22;
+  schatten_coeffs<Dual<T>>(Da, Db, Dc, Dt, a.sp, A11, A12, A22);
   const T s4 = group_sum<G>(kok ? v4 : T(0));
   // ---- adjoints of the outputs: wbar^k = G bbar, dbar^k = -vbar^{k+1}
   const T nd1 = a.vn_loc && kok ? a.vn_loc[el] : T(0);
@@ -195,10 +197,11 @@ __global__ void __launch_bounds__(ADJ_THREADS, 2) k_adj_vjp(const AdjArgs<T> a) 
   // block 1 (data term): ubar1 = 2 bbar - vbar1^{k+1}
   const T ub1 = T(2) * bc - nd1;
   const T su = group_sum<G>(kok ? ub1 * pk : T(0));
-  const T vb1 = -bc + nd1 + (ub1 - su * pk / (a.mu * t * disc));
+  const T vb1 = -bc + nd1 + (ub1 - su * pk * (imt * idisc));
   if (kok) {
-    const T dtdp = (a.mu * v1 * t + T(2) * pk) / (a.mu * disc);
-    const T pbar = ub1 / (a.mu * t) - su / (a.mu * t * t) * dtdp;
+    // dt/dp = (mu v1 t + 2 p) / (mu disc), pbar = ubar / (mu t) - su / (mu t^2) dt/dp
+    const T dtdp = (v1 + T(2) * pk * imt) * t * idisc;
+    const T pbar = (ub1 - su * (a.mu * imt) * dtdp) * imt;
     a.glogp[e] += pk * pbar;
   }
   // block 3 (positive orthant) and block 4 (affine set, or the probability simplex)
@@ -250,8 +253,10 @@ __global__ void __launch_bounds__(ADJ_THREADS, 2) k_adj_vjp(const AdjArgs<T> a) 
   }
   Ab11 = group_sum<G>(Ab11); Ab12 = group_sum<G>(Ab12); Ab22 = group_sum<G>(Ab22);
   T gbar4[4];
+  const T gtan = Ab11 * A11.d + Ab12 * A12.d + Ab22 * A22.d;
 #pragma unroll
-  for (int m = 0; m < 4; ++m) gbar4[m] = Ab11 * A11.d[m] + Ab12 * A12.d[m] + Ab22 * A22.d[m];
+  for (int m = 0; m < 4; ++m) gbar4[m] = __shfl_sync(0xffffffffu, gtan, m, G);
+  const T C11 = T(2) * A11.v - T(1), C12 = T(2) * A12.v, C22 = T(2) * A22.v - T(1);  // w2 = V (2A - I)
   // per-thread terms of the parameter gradients, in the working precision (FP64 only from the
   // warp sums on: FP64 arithmetic is scarce on this part)
   T om_loc[L];
@@ -274,10 +279,8 @@ __global__ void __launch_bounds__(ADJ_THREADS, 2) k_adj_vjp(const AdjArgs<T> a) 
     if (kok) st_pair(a.v_2 + e2 + (size_t)j * K * 2, vbh, vbv);
     // omega_j: v2 = omega_j S_j D z^k - d2 (first term); b = G^T w with w2 = 2 u2 - v2 (second)
     const T zdh = zw[dy][dx + 1] - zw[dy][dx], zdv = zw[dy + 1][dx] - zw[dy][dx];
-    const T u2h = vh[j] * A11.v + vv[j] * A12.v, u2v = vh[j] * A12.v + vv[j] * A22.v;
-    om_loc[j] = kok ? (vbh * zdh + vbv * zdv) +
-                          (jbh[j] * (T(2) * u2h - vh[j]) + jbv[j] * (T(2) * u2v - vv[j]))
-                    : T(0);
+    const T w2h = vh[j] * C11 + vv[j] * C12, w2v = vh[j] * C12 + vv[j] * C22;
+    om_loc[j] = kok ? (vbh * zdh + vbv * zdv) + (jbh[j] * w2h + jbv[j] * w2v) : T(0);
   }
   if (kok) {
     a.v_loc[el] = vb1;
@@ -289,27 +292,39 @@ __global__ void __launch_bounds__(ADJ_THREADS, 2) k_adj_vjp(const AdjArgs<T> a) 
     const T z1 = a.zk1[e];
     s_loc = (a.bbar[qh] - bc) * (a.zk1[qh] - z1) + (a.bbar[qv] - bc) * (a.zk1[qv] - z1);
   }
-  // block partial sums (tau once per pixel, from lane 0): warp shuffles in the working
-  // precision, then the warps in a fixed order in FP64 (deterministic)
+  // block partial sums (tau once per pixel, from lane 0): over each warp in the working precision,
+  // then the warps in a fixed order in FP64 (deterministic). The warp sums of all parameters
+  // together: at each halving a lane hands over half of its values and adds its partner's half of
+  // the ones it keeps, NV + 1 additions or so for NV values instead of 5 NV
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  auto wsum = [&](T v) {
+  constexpr int NV = NP <= 4 ? 4 : NP <= 16 ? 16 : 32;   // values, padded to a power of two
+  T v[NV];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-  };
-  {
-    const T t0 = wsum((pok && g == 0) ? gbar4[3] : T(0));
-    if (lane == 0) red[warp][0] = (double)t0;
-  }
+  for (int j = 0; j < NV; ++j) v[j] = T(0);
+  v[0] = (pok && g == 0) ? gbar4[3] : T(0);
 #pragma unroll
-  for (int j = 0; j < L; ++j) {
-    const T t1 = wsum(om_loc[j]);
-    if (lane == 0) red[warp][1 + j] = (double)t1;
+  for (int j = 0; j < L; ++j) v[1 + j] = om_loc[j];
+  v[L + 1] = s_loc;
+  int nv = NV, off = 16, at = 0;                  // lane's values are v[at .. at + nv) of the original
+#pragma unroll
+  for (int lv = 0; lv < 5; ++lv, off >>= 1) {
+    const bool upper = (lane & off) != 0;
+    if (nv > 1) {
+      nv >>= 1;
+#pragma unroll
+      for (int j = 0; j < NV / 2; ++j) {
+        if (j < nv) {
+          const T keep = upper ? v[j + nv] : v[j], give = upper ? v[j] : v[j + nv];
+          v[j] = keep + __shfl_xor_sync(0xffffffffu, give, off);
+        }
+      }
+      at += upper ? nv : 0;
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+    }
   }
-  {
-    const T t2 = wsum(s_loc);
-    if (lane == 0) red[warp][L + 1] = (double)t2;
-  }
+  // lanes that differ only in the last (plain) halvings hold the same sum
+  if ((lane & (32 / NV - 1)) == 0 && at < NP) red[warp][at] = (double)v[0];
   __syncthreads();
   for (int j = threadIdx.x; j < NP; j += blockDim.x) {
     double t = 0.0;

@@ -36,6 +36,7 @@ enum Kind { KIND_SWEEP = 0, KIND_ROWF = 1, KIND_COL = 2, KIND_ROWI = 3, KIND_DIA
             KIND_MLR = 6, KIND_ADJ = 7, KIND_ZF = 8 };
 constexpr int NKIND = 9;
 constexpr int MAXCOV = 2;           // tile covers per row / column in the partial gather
+constexpr size_t ADJ_KEEP_BYTES = size_t(64) << 20;  // largest reverse-pass memory a handle keeps
 constexpr int TRACE_CAP = 128;      // device trace records before a flush to the host
 // Images from this many pixels up run the pipelined row passes unless the tiling says otherwise.
 constexpr long long ROWPIPE_DEFAULT_PIXELS = 1LL << 62;
@@ -539,6 +540,8 @@ class Solver : public SolverBase {
   // the local duals are held in compact form (b.dcmp, written by the affine fused sweep)
   // rather than in full form (b.dloc: set_probs, set_state, the simplex and wide sweeps)
   bool dl_cmp = false;
+  // where the next sweep puts the new d2 and (simplex) full local duals; nullptr: in place
+  T *sweep_d2o = nullptr, *sweep_dloco = nullptr;
   bool p_quads = false;    // layout of the last sweep's rhs partials (see p_strides)
 
   // The form of the local duals the handle's sweeps keep from iteration to iteration (graphs
@@ -562,6 +565,8 @@ class Solver : public SolverBase {
   double* trace_host = nullptr;  // pinned staging for trace records
   void* mlr_buf = nullptr;       // device staging of host spectra / weights / biases
   size_t mlr_cap = 0;
+  void* adj_buf = nullptr;       // memory of small reverse passes (adj_memory)
+  size_t adj_cap = 0;
   int trace_host_cap = 0;
   bool use_graphs = true;
   int g4 = SEGSALSA_G4_AFFINE;   // MPO of g4: affine set (eq. 10) or probability simplex
@@ -575,6 +580,7 @@ class Solver : public SolverBase {
       if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
     if (trace_host) cudaFreeHost(trace_host);
     if (mlr_buf) cudaFree(mlr_buf);
+    if (adj_buf) cudaFree(adj_buf);
     for (auto& e : evs) { cudaEventDestroy(std::get<1>(e)); cudaEventDestroy(std::get<2>(e)); }
     for (auto e : evpool) cudaEventDestroy(e);
     if (own_ws && ws) cudaFree(ws);
@@ -647,57 +653,28 @@ class Solver : public SolverBase {
   }
 
   int upload_tables() {
-    const int H = pl.H, W = pl.W, Wh = pl.Wh, Mf = pl.Mf;
-    std::vector<T> om(pl.L);
-    for (int j = 0; j < pl.L; ++j) om[j] = (T)omega[j];
-    SGS_CUDA(cudaMemcpyAsync(b.omega, om.data(), sizeof(T) * pl.L, cudaMemcpyHostToDevice, st));
+    const int W = pl.W, Mf = pl.Mf;
     SGS_CUDA(cudaMemsetAsync(b.err, 0, sizeof(int), st));
     SGS_CUDA(cudaMemsetAsync(b.zctr, 0, 4 * sizeof(unsigned int), st));
     SGS_CUDA(cudaMemcpyAsync(b.covY, pl.covY.data(), sizeof(int) * pl.covY.size(), cudaMemcpyHostToDevice, st));
     SGS_CUDA(cudaMemcpyAsync(b.covX, pl.covX.data(), sizeof(int) * pl.covX.size(), cudaMemcpyHostToDevice, st));
+    std::vector<int> off(pl.covX.size()), offq;
     {
-      std::vector<int> off(pl.covX.size());
       for (size_t i = 0; i < off.size(); ++i) {
         const int cx = pl.covX[i];
         off[i] = cx < 0 ? -1 : ((cx >> 16) * pl.EHmax * pl.EWmax + (cx & 0xffff)) * pl.K;
       }
       SGS_CUDA(cudaMemcpyAsync(b.offX, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice, st));
-      SGS_CUDA(cudaStreamSynchronize(st));  // `off` leaves scope
       if (pl.zl) {
-        off.assign(pl.covY.size(), -1);
-        for (size_t i = 0; i < off.size(); ++i) {
+        offq.assign(pl.covY.size(), -1);
+        for (size_t i = 0; i < offq.size(); ++i) {
           const int cy = pl.covY[i];
           if (cy >= 0)
-            off[i] = ((cy >> 16) * pl.ntx * ((pl.K + 3) / 4) * pl.EHmax + (cy & 0xffff)) * pl.EWmax;
+            offq[i] = ((cy >> 16) * pl.ntx * ((pl.K + 3) / 4) * pl.EHmax + (cy & 0xffff)) * pl.EWmax;
         }
-        SGS_CUDA(cudaMemcpyAsync(b.offYq, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice, st));
-        SGS_CUDA(cudaStreamSynchronize(st));
+        SGS_CUDA(cudaMemcpyAsync(b.offYq, offq.data(), sizeof(int) * offq.size(), cudaMemcpyHostToDevice, st));
       }
     }
-    // column solve coefficients, per kx: (a + 2c) - c (S + S^-1) = (c/beta)(1 - beta S)(1 - beta/S)
-    std::vector<T> beta(Wh), gain(Wh), wfac(Wh);
-    std::vector<int> nwarm(Wh);
-    const double tol = sizeof(T) == 4 ? 1e-9 : 1e-18;
-    const double c = c_omega;
-    for (int kx = 0; kx < Wh; ++kx) {
-      const double s = std::sin(M_PI * kx / W);
-      const double alpha = 3.0 + c * (4.0 * s * s + 2.0);
-      if (c > 0.0) {
-        const double t = alpha / c;
-        const double bt = 2.0 / (t + std::sqrt(t * t - 4.0));
-        const double gn = 2.0 / (alpha + std::sqrt(alpha * alpha - 4.0 * c * c));
-        int nw = (int)std::ceil(std::log(tol * (1.0 - bt)) / std::log(bt));
-        double wf = 1.0;
-        if (nw >= H || nw < 0) { nw = H; wf = 1.0 / (1.0 - std::pow(bt, H)); }
-        beta[kx] = (T)bt; gain[kx] = (T)gn; wfac[kx] = (T)wf; nwarm[kx] = nw;
-      } else {
-        beta[kx] = 0; gain[kx] = (T)(1.0 / alpha); wfac[kx] = 1; nwarm[kx] = 0;
-      }
-    }
-    SGS_CUDA(cudaMemcpyAsync(b.beta, beta.data(), sizeof(T) * Wh, cudaMemcpyHostToDevice, st));
-    SGS_CUDA(cudaMemcpyAsync(b.gain, gain.data(), sizeof(T) * Wh, cudaMemcpyHostToDevice, st));
-    SGS_CUDA(cudaMemcpyAsync(b.wfac, wfac.data(), sizeof(T) * Wh, cudaMemcpyHostToDevice, st));
-    SGS_CUDA(cudaMemcpyAsync(b.nwarm, nwarm.data(), sizeof(int) * Wh, cudaMemcpyHostToDevice, st));
     // FFT tables (FP64 on the host)
     std::vector<cplx<T>> tw(Mf), chirp(W), bhat(Mf);
     for (int m = 0; m < Mf; ++m) {
@@ -731,6 +708,39 @@ class Solver : public SolverBase {
     SGS_CUDA(cudaMemcpyAsync(b.tw, tw.data(), sizeof(cplx<T>) * Mf, cudaMemcpyHostToDevice, st));
     SGS_CUDA(cudaMemcpyAsync(b.chirp, chirp.data(), sizeof(cplx<T>) * W, cudaMemcpyHostToDevice, st));
     SGS_CUDA(cudaMemcpyAsync(b.bhat, bhat.data(), sizeof(cplx<T>) * Mf, cudaMemcpyHostToDevice, st));
+    return upload_weights();    // synchronizes before the host arrays leave scope
+  }
+
+  // The tables that depend on the shift weights: the weights and the column solve's coefficients.
+  int upload_weights() {
+    const int H = pl.H, W = pl.W, Wh = pl.Wh;
+    std::vector<T> om(pl.L);
+    for (int j = 0; j < pl.L; ++j) om[j] = (T)omega[j];
+    SGS_CUDA(cudaMemcpyAsync(b.omega, om.data(), sizeof(T) * pl.L, cudaMemcpyHostToDevice, st));
+    // column solve coefficients, per kx: (a + 2c) - c (S + S^-1) = (c/beta)(1 - beta S)(1 - beta/S)
+    std::vector<T> beta(Wh), gain(Wh), wfac(Wh);
+    std::vector<int> nwarm(Wh);
+    const double tol = sizeof(T) == 4 ? 1e-9 : 1e-18;
+    const double c = c_omega;
+    for (int kx = 0; kx < Wh; ++kx) {
+      const double s = std::sin(M_PI * kx / W);
+      const double alpha = 3.0 + c * (4.0 * s * s + 2.0);
+      if (c > 0.0) {
+        const double t = alpha / c;
+        const double bt = 2.0 / (t + std::sqrt(t * t - 4.0));
+        const double gn = 2.0 / (alpha + std::sqrt(alpha * alpha - 4.0 * c * c));
+        int nw = (int)std::ceil(std::log(tol * (1.0 - bt)) / std::log(bt));
+        double wf = 1.0;
+        if (nw >= H || nw < 0) { nw = H; wf = 1.0 / (1.0 - std::pow(bt, H)); }
+        beta[kx] = (T)bt; gain[kx] = (T)gn; wfac[kx] = (T)wf; nwarm[kx] = nw;
+      } else {
+        beta[kx] = 0; gain[kx] = (T)(1.0 / alpha); wfac[kx] = 1; nwarm[kx] = 0;
+      }
+    }
+    SGS_CUDA(cudaMemcpyAsync(b.beta, beta.data(), sizeof(T) * Wh, cudaMemcpyHostToDevice, st));
+    SGS_CUDA(cudaMemcpyAsync(b.gain, gain.data(), sizeof(T) * Wh, cudaMemcpyHostToDevice, st));
+    SGS_CUDA(cudaMemcpyAsync(b.wfac, wfac.data(), sizeof(T) * Wh, cudaMemcpyHostToDevice, st));
+    SGS_CUDA(cudaMemcpyAsync(b.nwarm, nwarm.data(), sizeof(int) * Wh, cudaMemcpyHostToDevice, st));
     SGS_CUDA(cudaStreamSynchronize(st));
     return SEGSALSA_OK;
   }
@@ -796,10 +806,14 @@ class Solver : public SolverBase {
   // Bring the full form up to date (d1 = c1 p, d4 = c4 1) and make it the one in use.
   int dl_to_full() {
     if (!dl_cmp) return SEGSALSA_OK;
+    if (int rc = dl_expand(b.dloc)) return rc;
+    dl_cmp = false;
+    return SEGSALSA_OK;
+  }
+  int dl_expand(T* dst) {
     const size_t nK = (size_t)pl.n * pl.K;
     const int blocks = (int)std::min<size_t>((nK + AUX_THREADS - 1) / AUX_THREADS, 152 * 8);
-    SGS_LAUNCH(KIND_OTHER, (k_dl_expand<T><<<blocks, AUX_THREADS, 0, st>>>(b.dcmp, b.p, b.dloc, pl.n, pl.K)));
-    dl_cmp = false;
+    SGS_LAUNCH(KIND_OTHER, (k_dl_expand<T><<<blocks, AUX_THREADS, 0, st>>>(b.dcmp, b.p, dst, pl.n, pl.K)));
     return SEGSALSA_OK;
   }
 
@@ -914,6 +928,8 @@ class Solver : public SolverBase {
     a.H = pl.H; a.W = pl.W; a.K = pl.K; a.NC = pl.NC; a.ntx = pl.ntx; a.nty = pl.nty;
     a.EHmax = pl.EHmax; a.EWmax = pl.EWmax;
     a.z = b.z; a.p = b.p; a.dloc = b.dloc; a.d2 = b.d2; a.P = b.P; a.P2 = b.P2;
+    a.d2o = sweep_d2o ? sweep_d2o : b.d2;
+    a.dloco = sweep_dloco ? sweep_dloco : b.dloc;
     a.dcmp = b.dcmp;
     p_quads = zl_now();
     p_strides(p_quads, a.pstr, a.pquad, a.ptile);
@@ -1441,6 +1457,7 @@ class Solver : public SolverBase {
 
   int set_lambda(double lam) override {
     if (!(lam >= 0.0) || !std::isfinite(lam)) return fail(SEGSALSA_ERR_ARG, "lambda must be finite and >= 0");
+    if (lam == lambda) return SEGSALSA_OK;
     SGS_CUDA(cudaStreamSynchronize(st));
     lambda = lam;
     drop_chunks();
@@ -1451,12 +1468,35 @@ class Solver : public SolverBase {
     if (!w) return fail(SEGSALSA_ERR_ARG, "weights is NULL");
     for (int j = 0; j < pl.L; ++j)
       if (!std::isfinite(w[j])) return fail(SEGSALSA_ERR_ARG, "weights must be finite");
+    if (std::equal(omega.begin(), omega.end(), w)) return SEGSALSA_OK;
     SGS_CUDA(cudaStreamSynchronize(st));
     for (int j = 0; j < pl.L; ++j) omega[j] = w[j];
     c_omega = 0.0;
     for (double v : omega) c_omega += v * v;
     drop_chunks();
-    return upload_tables();
+    return upload_weights();
+  }
+
+  // Device memory of a reverse pass: kept by the handle while it is small (an allocation and its
+  // release cost a short pass more than its kernels), else allocated for the call (the caller frees
+  // it when it is not adj_buf).
+  int adj_memory(size_t bytes, void** mem) {
+    cudaError_t e = cudaSuccess;
+    if (bytes > ADJ_KEEP_BYTES) {
+      e = cudaMalloc(mem, bytes);
+    } else {
+      if (bytes > adj_cap) {
+        if (adj_buf) cudaFree(adj_buf);
+        adj_buf = nullptr;
+        adj_cap = 0;
+        e = cudaMalloc(&adj_buf, bytes);
+        if (e == cudaSuccess) adj_cap = bytes;
+        else adj_buf = nullptr;
+      }
+      *mem = adj_buf;
+    }
+    if (e != cudaSuccess) return fail(SEGSALSA_ERR_OOM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+    return SEGSALSA_OK;
   }
 
   // Reverse pass of `iters` iterations from the current p (see adjoint.cuh for the algebra).
@@ -1475,15 +1515,16 @@ class Solver : public SolverBase {
     const int nseg = (iters + every - 1) / every;
     const int blocks = (n + ADJ_THREADS / pl.G - 1) / (ADJ_THREADS / pl.G);
     const size_t npart = (size_t)blocks * (L + 2);
-    // device memory of the pass (released at the end)
+    // device memory of the pass: a checkpoint for every segment but the last, whose states the
+    // forward pass leaves in the segment's slots; one segment's states; the final partials
     Carver cv{nullptr};
     auto plan = [&](Carver& c, T*& ck, T*& fin, T*& zs, T*& dls, T*& d2s, T*& vbl, T*& vb2,
                     T*& zb, T*& bb, T*& glp, double*& part, double*& acc) {
-      ck = c.take<T>((size_t)nseg * st_elems);
-      fin = c.take<T>(st_elems);
+      ck = c.take<T>((size_t)(nseg - 1) * st_elems);
+      fin = c.take<T>(nseg > 1 ? tslot : 0);
       zs = c.take<T>((size_t)(every + 2) * nK);
-      dls = c.take<T>((size_t)(every + 1) * nloc);
-      d2s = c.take<T>((size_t)(every + 1) * n2);
+      dls = c.take<T>((size_t)(every + 1) * nloc + 64 / sizeof(T));
+      d2s = c.take<T>((size_t)(every + 1) * n2 + 64 / sizeof(T));
       vbl = c.take<T>(2 * nloc);   // vbar local blocks, two buffers
       vb2 = c.take<T>(2 * n2);     // vbar d2 blocks, two buffers (pairs stay 2 T aligned)
       zb = c.take<T>(nK);
@@ -1496,28 +1537,53 @@ class Solver : public SolverBase {
     double *part, *acc;
     plan(cv, ck, fin, zs, dls, d2s, vbl, vb2, zb, bb, glp, part, acc);
     void* mem = nullptr;
-    cudaError_t e = cudaMalloc(&mem, cv.off);
-    if (e != cudaSuccess) return fail(SEGSALSA_ERR_OOM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
-    struct Free { void* m; ~Free() { cudaFree(m); } } guard{mem};
+    if (int rc = adj_memory(cv.off, &mem)) return rc;
+    struct Free { void* m; ~Free() { if (m) cudaFree(m); } } guard{mem == adj_buf ? nullptr : mem};
     Carver cm{static_cast<char*>(mem)};
     plan(cm, ck, fin, zs, dls, d2s, vbl, vb2, zb, bb, glp, part, acc);
-    auto save = [&](T* dst) -> cudaError_t {
-      cudaError_t r;
-      if (dl_to_full()) return cudaErrorUnknown;   // checkpoints hold the full form
-      if ((r = cudaMemcpyAsync(dst, b.z, sizeof(T) * nK, cudaMemcpyDeviceToDevice, st))) return r;
-      if ((r = cudaMemcpyAsync(dst + nK, b.dloc, sizeof(T) * nloc, cudaMemcpyDeviceToDevice, st))) return r;
-      if ((r = cudaMemcpyAsync(dst + nK + nloc, b.d2, sizeof(T) * n2, cudaMemcpyDeviceToDevice, st))) return r;
-      return cudaMemcpyAsync(dst + nK + nloc + n2, b.P, sizeof(T) * tslot, cudaMemcpyDeviceToDevice, st);
+    // the handle's own buffers come back on every way out
+    struct Restore {
+      Solver* s;
+      Buffers<T> keep;
+      ~Restore() { s->b = keep; s->sweep_d2o = s->sweep_dloco = nullptr; }
+    } restore{this, b};
+    const Buffers<T> own = b;
+    auto copy = [&](T* dst, const T* src, size_t count) {
+      return cudaMemcpyAsync(dst, src, sizeof(T) * count, cudaMemcpyDeviceToDevice, st);
     };
-    auto load = [&](const T* src) -> cudaError_t {
-      cudaError_t r;
-      if ((r = cudaMemcpyAsync(b.z, src, sizeof(T) * nK, cudaMemcpyDeviceToDevice, st))) return r;
-      if ((r = cudaMemcpyAsync(b.dloc, src + nK, sizeof(T) * nloc, cudaMemcpyDeviceToDevice, st))) return r;
-      dl_cmp = false;
-      if ((r = cudaMemcpyAsync(b.d2, src + nK + nloc, sizeof(T) * n2, cudaMemcpyDeviceToDevice, st))) return r;
-      return cudaMemcpyAsync(b.P, src + nK + nloc + n2, sizeof(T) * tslot, cudaMemcpyDeviceToDevice, st);
-    };
+    const bool simplex = g4 == SEGSALSA_G4_SIMPLEX;
     int rc;
+    // Iterations k0 .. k1 with the states kept: slot i of (zs, dls, d2s) holds z^k, d^k, k = k0 + i,
+    // slot 0 filled by the caller, b.P the partials of state k0. Every kernel reads one slot and
+    // writes the next. z^{k1+1} follows in its slot; d^{k1+1} goes to the handle's own buffers if
+    // `last` (the final state).
+    auto run_segment = [&](int k0, int k1, bool last) -> int {
+      b.z = zs; b.dloc = dls; b.d2 = d2s;
+      dl_cmp = false;
+      iter = k0;
+      rhs_dense = false;
+      for (int k = k0; k <= k1; ++k) {
+        const int i = k - k0;
+        T* zn = zs + (size_t)(i + 1) * nK;
+        if (k > 0) {
+          if ((rc = z_update(nullptr, zn))) return rc;
+        } else {
+          SGS_CUDA(copy(zn, b.z, nK));            // z^1 = z^0
+        }
+        b.z = zn;
+        if (k == k1 && !last) break;
+        sweep_d2o = k == k1 ? own.d2 : d2s + (size_t)(i + 1) * n2;
+        sweep_dloco = k == k1 ? own.dloc : dls + (size_t)(i + 1) * nloc;
+        if ((rc = sweep(false))) return rc;
+        b.d2 = sweep_d2o;
+        b.dloc = sweep_dloco;
+        // the reverse units read the full form
+        if (!simplex && (rc = dl_expand(b.dloc))) return rc;
+        iter = k + 1;
+      }
+      sweep_d2o = sweep_dloco = nullptr;
+      return SEGSALSA_OK;
+    };
     // forward from z^0 = p / 1^T p, d^0 = 0, with a checkpoint every `every` iterations
     SGS_LAUNCH(KIND_OTHER, (k_init_z<T><<<grid1(n), AUX_THREADS, 0, st>>>(b.p, b.z, n, K)));
     SGS_CUDA(cudaMemsetAsync(b.dloc, 0, sizeof(T) * nloc, st));
@@ -1525,11 +1591,23 @@ class Solver : public SolverBase {
     SGS_CUDA(cudaMemsetAsync(b.d2, 0, sizeof(T) * n2, st));
     iter = 0;
     rhs_dense = false;
-    for (int k = 0; k < iters; k += every) {
-      SGS_CUDA(save(ck + (size_t)(k / every) * st_elems));
-      if ((rc = solve(std::min(every, iters - k), nullptr, 0, nullptr))) return rc;
+    for (int seg = 0; seg < nseg - 1; ++seg) {
+      T* dst = ck + (size_t)seg * st_elems;
+      if ((rc = dl_to_full())) return rc;         // checkpoints hold the full form
+      SGS_CUDA(copy(dst, b.z, nK));
+      SGS_CUDA(copy(dst + nK, b.dloc, nloc));
+      SGS_CUDA(copy(dst + nK + nloc, b.d2, n2));
+      SGS_CUDA(copy(dst + nK + nloc + n2, b.P, tslot));
+      if ((rc = solve(every, nullptr, 0, nullptr))) return rc;
     }
-    SGS_CUDA(save(fin));
+    if ((rc = dl_to_full())) return rc;
+    SGS_CUDA(copy(zs, b.z, nK));
+    SGS_CUDA(copy(dls, b.dloc, nloc));
+    SGS_CUDA(copy(d2s, b.d2, n2));
+    if ((rc = run_segment((nseg - 1) * every, iters - 1, true))) return rc;
+    // the final z and duals stay in the handle's buffers, the partials are kept from recomputation
+    SGS_CUDA(copy(own.z, b.z, nK));
+    if (nseg > 1) SGS_CUDA(copy(fin, b.P, tslot));
     // seed: zbar^T, pixel-major
     if (layout == SEGSALSA_LAYOUT_HWK) {
       if ((rc = copy_in(zb, zbar, nK, dev))) return rc;
@@ -1546,22 +1624,14 @@ class Solver : public SolverBase {
       const int k0 = seg * every;
       const int k1 = std::min(k0 + every, iters - 1);
       if (k1 < k0 + 1) continue;                              // no unit in this segment
-      // recompute z^k, d^k (k0 <= k <= k1) and z^{k1+1} from the checkpoint
-      SGS_CUDA(load(ck + (size_t)seg * st_elems));
-      iter = k0;
-      rhs_dense = false;
-      for (int k = k0; k <= k1; ++k) {
-        const int i = k - k0;
-        SGS_CUDA(cudaMemcpyAsync(zs + (size_t)i * nK, b.z, sizeof(T) * nK, cudaMemcpyDeviceToDevice, st));
-        if ((rc = dl_to_full())) return rc;           // the reverse units read the full form
-        SGS_CUDA(cudaMemcpyAsync(dls + (size_t)i * nloc, b.dloc, sizeof(T) * nloc, cudaMemcpyDeviceToDevice, st));
-        SGS_CUDA(cudaMemcpyAsync(d2s + (size_t)i * n2, b.d2, sizeof(T) * n2, cudaMemcpyDeviceToDevice, st));
-        if (k < k1) {
-          if ((rc = iteration(false, 0))) return rc;
-        } else {
-          if ((rc = z_update(nullptr, b.z))) return rc;         // z^{k1+1} (k1 >= 1)
-          SGS_CUDA(cudaMemcpyAsync(zs + (size_t)(i + 1) * nK, b.z, sizeof(T) * nK, cudaMemcpyDeviceToDevice, st));
-        }
+      if (seg < nseg - 1) {
+        // recompute z^k, d^k (k0 <= k <= k1) and z^{k1+1} from the checkpoint
+        const T* src = ck + (size_t)seg * st_elems;
+        SGS_CUDA(copy(zs, src, nK));
+        SGS_CUDA(copy(dls, src + nK, nloc));
+        SGS_CUDA(copy(d2s, src + nK + nloc, n2));
+        SGS_CUDA(copy(b.P, src + nK + nloc + n2, tslot));
+        if ((rc = run_segment(k0, k1, false))) return rc;
       }
       // reverse units k1 .. k0+1
       for (int k = k1; k >= k0 + 1; --k) {
@@ -1588,6 +1658,7 @@ class Solver : public SolverBase {
         a.omega = b.omega;
         a.tau = (T)(lambda / mu);
         a.mu = (T)mu;
+        a.mu4 = (T)(4.0 / mu);
         a.invK = (T)(1.0 / K);
         a.sp = sp;
         a.simplex = g4 == SEGSALSA_G4_SIMPLEX ? 1 : 0;
@@ -1609,7 +1680,8 @@ class Solver : public SolverBase {
       if ((rc = copy_out(glogp, b.tmp, nK, dev))) return rc;
     }
     // the handle ends where the forward pass ended: iteration `iters`
-    SGS_CUDA(load(fin));
+    if (nseg > 1) SGS_CUDA(copy(own.P, fin, tslot));
+    dl_cmp = false;
     iter = iters;
     rhs_dense = false;
     std::vector<double> sums(L + 2);   // tau, omega_0..omega_{L-1}, S

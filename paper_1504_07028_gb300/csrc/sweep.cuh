@@ -39,6 +39,8 @@ struct SweepArgs {
   int cin;               // affine g4: the local duals come in compact form (else full form);
                          // the affine sweep writes the compact form, the simplex sweep the full
   T* d2;                 // [n][L][K][2]
+  T* d2o;                // the new d2 (d2 itself: in place)
+  T* dloco;              // simplex: the new full form (dloc itself: in place)
   T* P;                  // per tile: partial sums of G^T(u + d) over [EHmax][EWmax] pixels; class k of
                          // pixel q at q * pstr + (k / 4) * pquad + k % 4 of the tile's ptile values
   int pstr, pquad, ptile;  // K, 4, EHmax EWmax K: pixel-major; 4, 4 EHmax EWmax, ...: planes of
@@ -505,7 +507,7 @@ __global__ void __launch_bounds__(NT, sweep_min_blocks<T, M, DIAG, NT>()) k_swee
     }
     if constexpr (SIMP) {
       if (kok) {
-        T* dl = a.dloc + pix0 * 3 * K + (cc * 3 * K + g);
+        T* dl = a.dloco + pix0 * 3 * K + (cc * 3 * K + g);
         dl[0] = n1;
         dl[K] = n3;
         dl[2 * K] = n4;
@@ -529,7 +531,7 @@ __global__ void __launch_bounds__(NT, sweep_min_blocks<T, M, DIAG, NT>()) k_swee
       accW[E - 1][s] = T(0);
       if constexpr (DIAG) accW2[E - 1][s] = T(0);
     }
-    V2* d2w = reinterpret_cast<V2*>(a.d2) + pix0 * L * K + (cc * L * K + g);
+    V2* d2w = reinterpret_cast<V2*>(a.d2o) + pix0 * L * K + (cc * L * K + g);
 #pragma unroll
     for (int dy = -M; dy <= M; ++dy)
 #pragma unroll
