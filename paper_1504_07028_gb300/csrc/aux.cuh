@@ -2,6 +2,8 @@
 // traced diagnostics (primal / dual residual, objective (7) at the simplex projection).
 #pragma once
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "sweep.cuh"
 
@@ -389,22 +391,22 @@ __global__ void __launch_bounds__(AUX_THREADS) k_prior(const T* zp, const T* ome
 }
 
 template <typename T, int G>
-inline void launch_project(int blocks, cudaStream_t st, const T* z, const T* p, T* zp, int n,
+inline void launch_project(int blocks, int threads, cudaStream_t st, const T* z, const T* p, T* zp, int n,
                            int K, const T* P2, const T* gtd, const int* covY, const int* offX,
                            int W, int ntx, int EHmax, int EWmax, double* part) {
-  launch_pdl(k_project<T, G>, dim3(blocks), dim3(AUX_THREADS), 0, st, z, p, zp, n, K, P2, gtd,
+  launch_pdl(k_project<T, G>, dim3(blocks), dim3(threads), 0, st, z, p, zp, n, K, P2, gtd,
              covY, offX, W, ntx, EHmax, EWmax, part);
 }
 template <typename T>
-inline cudaError_t launch_project_g(int G, int blocks, cudaStream_t st, const T* z, const T* p,
+inline cudaError_t launch_project_g(int G, int blocks, int threads, cudaStream_t st, const T* z, const T* p,
                                     T* zp, int n, int K, const T* P2, const T* gtd,
                                     const int* covY, const int* offX, int W, int ntx, int EHmax,
                                     int EWmax, double* part) {
   switch (G) {
-    case 4: launch_project<T, 4>(blocks, st, z, p, zp, n, K, P2, gtd, covY, offX, W, ntx, EHmax, EWmax, part); break;
-    case 8: launch_project<T, 8>(blocks, st, z, p, zp, n, K, P2, gtd, covY, offX, W, ntx, EHmax, EWmax, part); break;
-    case 16: launch_project<T, 16>(blocks, st, z, p, zp, n, K, P2, gtd, covY, offX, W, ntx, EHmax, EWmax, part); break;
-    default: launch_project<T, 32>(blocks, st, z, p, zp, n, K, P2, gtd, covY, offX, W, ntx, EHmax, EWmax, part); break;
+    case 4: launch_project<T, 4>(blocks, threads, st, z, p, zp, n, K, P2, gtd, covY, offX, W, ntx, EHmax, EWmax, part); break;
+    case 8: launch_project<T, 8>(blocks, threads, st, z, p, zp, n, K, P2, gtd, covY, offX, W, ntx, EHmax, EWmax, part); break;
+    case 16: launch_project<T, 16>(blocks, threads, st, z, p, zp, n, K, P2, gtd, covY, offX, W, ntx, EHmax, EWmax, part); break;
+    default: launch_project<T, 32>(blocks, threads, st, z, p, zp, n, K, P2, gtd, covY, offX, W, ntx, EHmax, EWmax, part); break;
   }
   return cudaGetLastError();
 }
@@ -454,23 +456,30 @@ inline cudaError_t launch_prior(int M, int G, int blocks, cudaStream_t st, const
 }
 
 // One trace record (k, primal, dual, objective, min z, max |1^T z - 1|), reducing the block
-// partials in a fixed order: FT_THREADS threads each sum a strided subset in FP64 (four
-// independent chains, so that loads are in flight together: one warp took 79 us for the 16384
-// tile partials of a 2048 x 2048 image, bound by load latency), then a fixed shuffle tree per
-// warp and the warp results in warp order.
+// partials in a fixed order: the threads each sum a strided subset in FP64 (four independent
+// chains, so that loads are in flight together: one warp took 79 us for the 16384 tile partials of
+// a 2048 x 2048 image, bound by load latency), then a fixed shuffle tree per warp and the warp
+// results in warp order. One CTA, as many warps as there are partials for: the trees are FP64 work
+// on the CTA's one unit (145 x 145: 1024 threads 23 us, 128 threads 12 us).
 constexpr int FT_THREADS = 1024;
+inline int finalize_threads(int nsq, int nproj, int nprior) {
+  const int n = std::max(nsq, std::max(nproj, nprior));
+  int t = 64;
+  while (t < FT_THREADS && 4 * t < n) t *= 2;
+  return t;
+}
 
 __global__ void __launch_bounds__(FT_THREADS) k_finalize_trace(
     const double* sq, int nsq, const double* proj, int nproj, const double* prior, int nprior,
     double k, double mu, double lambda, double* rec) {
   __shared__ double red[6][FT_THREADS / 32];
-  const int t = threadIdx.x, l = t & 31, w = t >> 5;
+  const int t = threadIdx.x, l = t & 31, w = t >> 5, NT = blockDim.x;
   auto sum = [&](const double* v, int n, int stride, int off) {
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int i0 = t; i0 < n; i0 += 4 * FT_THREADS) {
+    for (int i0 = t; i0 < n; i0 += 4 * NT) {
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const int i = i0 + FT_THREADS * u;
+        const int i = i0 + NT * u;
         if (i < n) acc[u] += v[stride * i + off];
       }
     }
@@ -484,7 +493,7 @@ __global__ void __launch_bounds__(FT_THREADS) k_finalize_trace(
   v[3] = sum(prior, nprior, 1, 0);
   v[4] = 1e300;
   v[5] = 0.0;
-  for (int i = t; i < nproj; i += FT_THREADS) {
+  for (int i = t; i < nproj; i += NT) {
     v[4] = fmin(v[4], proj[4 * i]);
     v[5] = fmax(v[5], proj[4 * i + 1]);
   }
@@ -504,8 +513,9 @@ __global__ void __launch_bounds__(FT_THREADS) k_finalize_trace(
   __syncthreads();
   if (w == 0) {
     double x[6];
+    const bool in = l < NT / 32;
 #pragma unroll
-    for (int q = 0; q < 6; ++q) x[q] = red[q][l];
+    for (int q = 0; q < 6; ++q) x[q] = in ? red[q][l] : (q == 4 ? 1e300 : 0.0);
     tree(x);
     if (l == 0) {
       rec[0] = k;

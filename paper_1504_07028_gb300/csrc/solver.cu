@@ -161,7 +161,7 @@ struct Plan {
   int zl;
   ZlPlan zlp;
   size_t pslot;            // values of the rhs partials (class quads padded where zl)
-  int nproj_blk, nprior_blk;
+  int nproj_blk, nproj_threads, nprior_blk;
   // wide patches (M >= 3): two-launch sweep (gram + transpose tiles) writing a dense rhs
   int wide, wntx1, wntiles1, wnblk2;
   std::vector<int> covY, covX;  // [H][MAXCOV], [W][MAXCOV]
@@ -433,7 +433,8 @@ static int make_plan(const segsalsa_str_params* pr, Plan& pl, std::string& msg,
   // round per block up to eight blocks per SM, grid-stride rounds beyond (small images need
   // every SM: four rounds per block left 20 blocks for 145 x 145, 27 instead of 15 us)
   const int cap = 152 * 8;
-  pl.nproj_blk = std::max(1, std::min(cap, (pl.n + AUX_THREADS - 1) / AUX_THREADS));
+  pl.nproj_threads = pl.n < 152 * AUX_THREADS ? 64 : AUX_THREADS;   // a block on every SM
+  pl.nproj_blk = std::max(1, std::min(cap, (pl.n + pl.nproj_threads - 1) / pl.nproj_threads));
   {
     const int pt = ((H + PRIOR_TH - 1) / PRIOR_TH) * ((W + PRIOR_TW - 1) / PRIOR_TW);
     pl.nprior_blk = std::max(1, std::min(cap, pt));
@@ -948,9 +949,11 @@ class Solver : public SolverBase {
 
   int diagnostics(int k, int rec) {
     const int n = pl.n, K = pl.K;
-    SGS_CUDA(launch(KIND_DIAG, [&]() { return launch_project_g<T>(pl.G, pl.nproj_blk, st, b.z, b.p, b.zp, n, K, (const T*)b.P2, pl.wide ? (const T*)b.P2 : nullptr, (const int*)b.covY, (const int*)b.offX, pl.W, pl.ntx, pl.EHmax, pl.EWmax, b.dproj); }));
+    SGS_CUDA(launch(KIND_DIAG, [&]() { return launch_project_g<T>(pl.G, pl.nproj_blk, pl.nproj_threads, st, b.z, b.p, b.zp, n, K, (const T*)b.P2, pl.wide ? (const T*)b.P2 : nullptr, (const int*)b.covY, (const int*)b.offX, pl.W, pl.ntx, pl.EHmax, pl.EWmax, b.dproj); }));
     SGS_CUDA(launch(KIND_DIAG, [&]() { return launch_prior<T>(pl.M, pl.G, pl.nprior_blk, st, b.zp, b.omega, pl.H, pl.W, K, sp, b.dprior); }));
-    SGS_CUDA(launch(KIND_DIAG, [&]() { return launch_pdl(k_finalize_trace, dim3(1), dim3(FT_THREADS), 0, st, (const double*)b.dsq, pl.wide ? pl.wntiles1 : pl.ntiles, (const double*)b.dproj, pl.nproj_blk, (const double*)b.dprior, pl.nprior_blk, (double)k, mu, lambda, b.dtrace + 6 * rec); }));
+    const int nsq = pl.wide ? pl.wntiles1 : pl.ntiles;
+    const int nt = finalize_threads(nsq, pl.nproj_blk, pl.nprior_blk);
+    SGS_CUDA(launch(KIND_DIAG, [&]() { return launch_pdl(k_finalize_trace, dim3(1), dim3(nt), 0, st, (const double*)b.dsq, nsq, (const double*)b.dproj, pl.nproj_blk, (const double*)b.dprior, pl.nprior_blk, (double)k, mu, lambda, b.dtrace + 6 * rec); }));
     return SEGSALSA_OK;
   }
 

@@ -195,6 +195,19 @@ template <typename T> struct Vec2Of;
 template <> struct Vec2Of<float> { using type = float2; };
 template <> struct Vec2Of<double> { using type = double2; };
 
+// A second read of a staged pair, as its own load (the traced sweep needs the old d2 twice and has no
+// registers to keep it).
+__device__ __forceinline__ float2 ld_shared_again(const float2* p) {
+  float2 v;
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(smem_addr(p)));
+  return v;
+}
+__device__ __forceinline__ double2 ld_shared_again(const double2* p) {
+  double2 v;
+  asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(smem_addr(p)));
+  return v;
+}
+
 // Byte sizes of one pipeline stage (one tile row of d2, dloc and p, each with 16 bytes of
 // alignment slack at both ends), for tiles at most NC pixels wide.
 __host__ __device__ inline size_t al16(size_t v) { return (v + 15) / 16 * 16; }
@@ -274,24 +287,28 @@ __device__ __forceinline__ void flush_sum(int c, int g, const T* slots, const T*
   }
 }
 
-// Warps an SM holds: 24 for the plain FP32 variant (80 registers, no spills); 16 otherwise.
-template <typename T, int M, bool DIAG, int NT>
-constexpr int sweep_min_blocks() { return ((sizeof(T) == 8 || M >= 2 || DIAG) ? 2 : 3) * (256 / NT); }
+// Warps an SM holds: 24 for the FP32 variants up to 3 x 3 (80 registers), 16 otherwise. The traced
+// ones take 80 registers only with compile-time class strides (2048 x 2048, K = 16: a trace costs 846 us
+// with 16 warps, 735 with 24; 400 x 300, K = 9: 55 against 69, its spills outweigh them).
+template <typename T, int M, bool DIAG, bool KEQ, int NT>
+constexpr int sweep_min_blocks() {
+  return ((sizeof(T) == 8 || M >= 2 || (DIAG && !KEQ)) ? 2 : 3) * (256 / NT);
+}
 
 // Flush slot buffers: two in FP32, so that one barrier a row orders them (and the stages); FP64 and
-// the simplex form, whose stages are larger, keep one and a second barrier.
-template <typename T, bool SIMP>
-constexpr int sweep_slot_bufs() { return (sizeof(T) == 4 && !SIMP) ? 2 : 1; }
+// the simplex and traced forms, whose stages or slots are larger, keep one and a second barrier.
+template <typename T, bool DIAG, bool SIMP>
+constexpr int sweep_slot_bufs() { return (sizeof(T) == 4 && !SIMP && !DIAG) ? 2 : 1; }
 
 // SIMP selects the MPO of g4: false, the projection onto the affine set 1^T xi = 1 (eq. 10);
 // true, the projection onto the probability simplex (Sec. 4's description of that MPO).
 // KEQ: the class count equals the lane count G, so the class strides are compile-time constants
 // (measured 8 % fewer sweep cycles at 145 x 145, K = 16). NT: threads of a CTA.
 template <typename T, int M, int G, bool DIAG, bool SIMP, bool KEQ, int NT>
-__global__ void __launch_bounds__(NT, sweep_min_blocks<T, M, DIAG, NT>()) k_sweep(const SweepArgs<T> a) {
+__global__ void __launch_bounds__(NT, sweep_min_blocks<T, M, DIAG, KEQ, NT>()) k_sweep(const SweepArgs<T> a) {
   constexpr int L = (2 * M + 1) * (2 * M + 1);
   constexpr int E = 2 * M + 2;
-  constexpr int SB = sweep_slot_bufs<T, SIMP>();
+  constexpr int SB = sweep_slot_bufs<T, DIAG, SIMP>();
   using V2 = typename Vec2Of<T>::type;
 
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -539,7 +556,8 @@ __global__ void __launch_bounds__(NT, sweep_min_blocks<T, M, DIAG, NT>()) k_swee
         const int j = (dy + M) * (2 * M + 1) + (dx + M);
         const T nh = vh[j] * B11 + vv[j] * B12, nv = vh[j] * B12 + vv[j] * B22;
         if constexpr (DIAG) {
-          const T eh = nh - dv[j].x, ev = nv - dv[j].y;
+          const V2 od = ld_shared_again(sd2 + j * K);
+          const T eh = nh - od.x, ev = nv - od.y;
           if (kok) sq += eh * eh + ev * ev;
         }
         if (kok) {
@@ -616,7 +634,7 @@ inline size_t sweep_smem_bytes(int nt, int NC, int EHmax, int EWmax, int G, int 
   size_t d2b, dlb, pb;
   stage_sizes<T>(NC, L, K, compact ? K + 2 : 3 * K, d2b, dlb, pb);
   const int E = EWmax - NC;  // 2M + 1 ... the window width is E + 1 = 2M + 2
-  const size_t slots = (size_t)(E + 1) * (nt / G + E) * G * (sizeof(T) == 4 && !simplex ? 2 : 1);
+  const size_t slots = (size_t)(E + 1) * (nt / G + E) * G * (sizeof(T) == 4 && !simplex && !diag ? 2 : 1);
   return 128 + 2 * (d2b + dlb + pb) +
          sizeof(T) * ((size_t)EHmax * EWmax * G + (size_t)((L + 3) & ~3) +
                       (diag ? 2 : 1) * slots);
