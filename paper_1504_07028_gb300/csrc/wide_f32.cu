@@ -5,20 +5,22 @@
 
 namespace sgs {
 
-template <int G, bool DIAG, bool SIMP>
+// one record per kernel: the type is part of its name, since the linker makes one object of equally
+// named ones in different files
+template <typename T, int G, bool DIAG, bool SIMP>
 struct WideGramGrant { static SmemGrants g; };
-template <int G, bool DIAG, bool SIMP> SmemGrants WideGramGrant<G, DIAG, SIMP>::g;
+template <typename T, int G, bool DIAG, bool SIMP> SmemGrants WideGramGrant<T, G, DIAG, SIMP>::g;
 
-template <int G, bool DIAG>
+template <typename T, int G, bool DIAG>
 struct WideJtGrant { static SmemGrants g; };
-template <int G, bool DIAG> SmemGrants WideJtGrant<G, DIAG>::g;
+template <typename T, int G, bool DIAG> SmemGrants WideJtGrant<T, G, DIAG>::g;
 
 template <int G, bool DIAG, bool SIMP>
 static cudaError_t wide_g(const WideArgs<float>& a, cudaStream_t st) {
   const size_t s1 = wide_gram_smem<float>(a.M, G), s2 = wide_jt_smem<float>(a.M, G);
-  cudaError_t e = grant_smem(k_wide_gram<float, G, DIAG, SIMP>, s1, WideGramGrant<G, DIAG, SIMP>::g);
+  cudaError_t e = grant_smem(k_wide_gram<float, G, DIAG, SIMP>, s1, WideGramGrant<float, G, DIAG, SIMP>::g);
   if (e != cudaSuccess) return e;
-  if ((e = grant_smem(k_wide_jt<float, G, DIAG>, s2, WideJtGrant<G, DIAG>::g)) != cudaSuccess) return e;
+  if ((e = grant_smem(k_wide_jt<float, G, DIAG>, s2, WideJtGrant<float, G, DIAG>::g)) != cudaSuccess) return e;
   if (st == reinterpret_cast<cudaStream_t>(-1)) return cudaSuccess;  // grants only
   if ((e = launch_pdl(k_wide_gram<float, G, DIAG, SIMP>, dim3(a.ntiles1), dim3(256), s1, st, a)) != cudaSuccess)
     return e;
