@@ -163,7 +163,7 @@ struct Plan {
   size_t pslot;            // values of the rhs partials (class quads padded where zl)
   int nproj_blk, nproj_threads, nprior_blk;
   // wide patches (M >= 3): two-launch sweep (gram + transpose tiles) writing a dense rhs
-  int wide, wntx1, wntiles1, wnblk2;
+  int wide, wntx1, wntiles1;
   std::vector<int> covY, covX;  // [H][MAXCOV], [W][MAXCOV]
 };
 
@@ -262,8 +262,6 @@ static int make_plan(const segsalsa_str_params* pr, Plan& pl, std::string& msg,
   pl.wide = M >= 3;
   pl.wntx1 = (W + 256 / pl.G - 1) / (256 / pl.G);
   pl.wntiles1 = pl.wntx1 * ((H + WG_TH - 1) / WG_TH);
-  // transpose: the gram tiles again (one row of 256 / G targets), at most 8 blocks per SM
-  pl.wnblk2 = std::max(1, std::min(152 * 8, pl.wntiles1));
   if (pl.wide) {
     if (wide_gram_smem<T>(M, pl.G) > 227 * 1024) {
       msg = "wide-patch tiles do not fit in shared memory"; return SEGSALSA_ERR_ARG;
@@ -913,7 +911,7 @@ class Solver : public SolverBase {
       w.rhs = b.rhsd;
       w.gtd = b.P2; w.diag_sq = b.dsq; w.omega = b.omega;
       w.tau = (T)(lambda / mu); w.mu = (T)mu; w.invK = (T)(1.0 / pl.K); w.sp = sp;
-      w.ntx1 = pl.wntx1; w.ntiles1 = pl.wntiles1; w.nblk2 = pl.wnblk2;
+      w.ntx1 = pl.wntx1; w.ntiles1 = pl.wntiles1;
       // three kernels per sweep (gram, shifted sums, differences); counted as sweep launches
       nlaunch[KIND_SWEEP] += 2;
       SGS_CUDA(launch(KIND_SWEEP, [&]() {

@@ -57,7 +57,6 @@ struct WideArgs {
   T tau, mu, invK;
   int sp;
   int ntx1, ntiles1; // gram tiles: columns of tiles, count
-  int nblk2;         // blocks of the transpose (grid-stride over pixels)
 };
 
 template <typename T>
@@ -84,8 +83,18 @@ __device__ __forceinline__ T prox_h(T vx, T vy, T a11, T a12) { return fma(vy, a
 template <typename T>
 __device__ __forceinline__ T prox_v(T vx, T vy, T a12, T a22) { return fma(vy, a22, vx * a12); }
 
+// CTAs of the Gram kernel an SM holds: its loads of V wait for DRAM, so registers are traded for warps
+// where a tile has few pixels (FP32, G >= 16: 48 registers and five CTAs against 59 and four, 512 x 512,
+// K = 16, 9 x 9 1414 -> 1368 us an iteration, while 64 x 64, K = 4 loses 1 %; a cap for six CTAs: 1414).
+// FP64 needs the bound of three stated: with one it takes 90 registers for 80 and an SM holds two
+// (145 x 145, K = 16, 7 x 7: 934 us against 918).
+template <typename T, int G, bool DIAG>
+constexpr int wide_gram_blocks() {
+  return sizeof(T) == 4 ? (G >= 16 && !DIAG ? 5 : 4) : DIAG ? 2 : 3;
+}
+
 template <typename T, int G, bool DIAG, bool SIMP>
-__global__ void __launch_bounds__(256) k_wide_gram(const WideArgs<T> a) {
+__global__ void __launch_bounds__(256, wide_gram_blocks<T, G, DIAG>()) k_wide_gram(const WideArgs<T> a) {
   constexpr int NC = 256 / G;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   T* zs = reinterpret_cast<T*>(smem_raw);
@@ -291,69 +300,69 @@ __global__ void __launch_bounds__(256) k_wide_jt(const WideArgs<T> a) {
     om[j] = a.omega[j];
   }
   pdl_wait();  // v, A and the local rhs come from k_wide_gram
-  for (int tile = blockIdx.x; tile < a.ntiles1; tile += gridDim.x) {
-    const int y = tile / a.ntx1, x0 = (tile % a.ntx1) * NC;
-    __syncthreads();  // the previous tile's window is no longer read
-    // A of the sources m - s_j of the tile's pixels (periodic)
-    for (int idx = threadIdx.x; idx < EHc * EWc; idx += blockDim.x) {
-      const int ry = idx / EWc, rx = idx - ry * EWc;
-      const int py = wrap_idx(y - M - 1 + ry, a.H), px = wrap_idx(x0 - M - 1 + rx, a.W);
-      T a11, a12, a22;
-      load_coef(a.coef, (size_t)py * a.W + px, a11, a12, a22);
-      cw[4 * idx] = a11;
-      cw[4 * idx + 1] = a12;
-      cw[4 * idx + 2] = a22;
-    }
-    __syncthreads();
-    const int x = x0 + c;
-    if (x >= a.W || g >= K) continue;   // no block-wide operation before the next tile's
-    const long long m = (long long)y * a.W + x;
-    const bool inner = y >= M && y <= a.H - 1 - M && x >= M && x <= a.W - 1 - M;
-    T sh = T(0), sv = T(0), dh = T(0), dv = T(0);
-    for (int j0 = 0; j0 < L; j0 += UJ) {
-      V2 v0[UJ];
+  // last tile first: the rows of V that the Gram pass wrote last are still in L2, and those read last
+  // here are the next Gram pass's first (145 x 145, K = 16, 9 x 9: 149.5 -> 143.4 us an iteration)
+  const int tile = a.ntiles1 - 1 - (int)blockIdx.x;
+  const int y = tile / a.ntx1, x0 = (tile % a.ntx1) * NC;
+  // A of the sources m - s_j of the tile's pixels (periodic)
+  for (int idx = threadIdx.x; idx < EHc * EWc; idx += blockDim.x) {
+    const int ry = idx / EWc, rx = idx - ry * EWc;
+    const int py = wrap_idx(y - M - 1 + ry, a.H), px = wrap_idx(x0 - M - 1 + rx, a.W);
+    T a11, a12, a22;
+    load_coef(a.coef, (size_t)py * a.W + px, a11, a12, a22);
+    cw[4 * idx] = a11;
+    cw[4 * idx + 1] = a12;
+    cw[4 * idx + 2] = a22;
+  }
+  __syncthreads();
+  const int x = x0 + c;
+  if (x >= a.W || g >= K) return;   // no block-wide operation follows
+  const long long m = (long long)y * a.W + x;
+  const bool inner = y >= M && y <= a.H - 1 - M && x >= M && x <= a.W - 1 - M;
+  T sh = T(0), sv = T(0), dh = T(0), dv = T(0);
+  for (int j0 = 0; j0 < L; j0 += UJ) {
+    V2 v0[UJ];
 #pragma unroll
-      for (int u = 0; u < UJ; ++u) {
-        const int j = j0 + u;
-        if (j >= L) break;
-        long long o0;
-        if (inner) {
-          o0 = m * LK + offv[j] + g;
-        } else {
-          int ys = y - dyx[2 * j], xs = x - dyx[2 * j + 1];   // m - s_j, periodic
-          ys += (ys < 0) ? a.H : 0;
-          ys -= (ys >= a.H) ? a.H : 0;
-          xs += (xs < 0) ? a.W : 0;
-          xs -= (xs >= a.W) ? a.W : 0;
-          o0 = (((long long)ys * a.W + xs) * L + j) * K + g;
-        }
-        v0[u] = vv2[o0];
+    for (int u = 0; u < UJ; ++u) {
+      const int j = j0 + u;
+      if (j >= L) break;
+      long long o0;
+      if (inner) {
+        o0 = m * LK + offv[j] + g;
+      } else {
+        int ys = y - dyx[2 * j], xs = x - dyx[2 * j + 1];   // m - s_j, periodic
+        ys += (ys < 0) ? a.H : 0;
+        ys -= (ys >= a.H) ? a.H : 0;
+        xs += (xs < 0) ? a.W : 0;
+        xs -= (xs >= a.W) ? a.W : 0;
+        o0 = (((long long)ys * a.W + xs) * L + j) * K + g;
       }
+      v0[u] = vv2[o0];
+    }
 #pragma unroll
-      for (int u = 0; u < UJ; ++u) {
-        const int j = j0 + u;
-        if (j >= L) break;
-        const Coef4<T> c0 = Coef4<T>::at(cw + woff[j] + 4 * c);
-        const T ux = prox_h(v0[u].x, v0[u].y, c0.a11, c0.a12);
-        const T uy = prox_v(v0[u].x, v0[u].y, c0.a12, c0.a22);
-        const T nx = ux - v0[u].x, ny = uy - v0[u].y;
-        const T o = om[j];
-        sh += o * (ux + nx);
-        sv += o * (uy + ny);
-        if constexpr (DIAG) {
-          dh += o * nx;
-          dv += o * ny;
-        }
+    for (int u = 0; u < UJ; ++u) {
+      const int j = j0 + u;
+      if (j >= L) break;
+      const Coef4<T> c0 = Coef4<T>::at(cw + woff[j] + 4 * c);
+      const T ux = prox_h(v0[u].x, v0[u].y, c0.a11, c0.a12);
+      const T uy = prox_v(v0[u].x, v0[u].y, c0.a12, c0.a22);
+      const T nx = ux - v0[u].x, ny = uy - v0[u].y;
+      const T o = om[j];
+      sh += o * (ux + nx);
+      sv += o * (uy + ny);
+      if constexpr (DIAG) {
+        dh += o * nx;
+        dv += o * ny;
       }
     }
-    const size_t oo = (size_t)m * K + g;
-    V2 r;
-    r.x = sh; r.y = sv;
-    S[oo] = r;
-    if constexpr (DIAG) {
-      r.x = dh; r.y = dv;
-      S[nK + oo] = r;
-    }
+  }
+  const size_t oo = (size_t)m * K + g;
+  V2 r;
+  r.x = sh; r.y = sv;
+  S[oo] = r;
+  if constexpr (DIAG) {
+    r.x = dh; r.y = dv;
+    S[nK + oo] = r;
   }
   pdl_trigger();
 }

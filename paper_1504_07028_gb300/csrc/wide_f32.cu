@@ -24,7 +24,7 @@ static cudaError_t wide_g(const WideArgs<float>& a, cudaStream_t st) {
   if (st == reinterpret_cast<cudaStream_t>(-1)) return cudaSuccess;  // grants only
   if ((e = launch_pdl(k_wide_gram<float, G, DIAG, SIMP>, dim3(a.ntiles1), dim3(256), s1, st, a)) != cudaSuccess)
     return e;
-  if ((e = launch_pdl(k_wide_jt<float, G, DIAG>, dim3(a.nblk2), dim3(256), s2, st, a)) != cudaSuccess)
+  if ((e = launch_pdl(k_wide_jt<float, G, DIAG>, dim3(a.ntiles1), dim3(256), s2, st, a)) != cudaSuccess)
     return e;
   const size_t nK = (size_t)a.H * a.W * a.K;
   const int nb3 = (int)std::min<size_t>((nK + 255) / 256, 152 * 8);
