@@ -215,7 +215,7 @@ int segsalsa_str_set_state(segsalsa_str_t* h, const void* z, const void* d1, con
                            int32_t on_device);
 
 /* The z-update operator alone: z = (3 I + J^T J)^{-1} rhs (eq. 12 with G^T G = 3I + J^T J),
- * rhs and z pixel-major (H, W, K). Leaves the solver state untouched. */
+ * rhs and z pixel-major (H, W, K); z may be rhs or overlap it. Leaves the solver state untouched. */
 int segsalsa_str_linear_solve(segsalsa_str_t* h, const void* rhs, void* z, int32_t on_device);
 
 /* Class model of the experiments (Sec. 5: the classes are modelled by a multinomial logistic

@@ -1304,9 +1304,17 @@ class Solver : public SolverBase {
       if ((rc = copy_in(b.tmp, rhs, nK, 0))) return rc;
       src = b.tmp;
     }
-    T* out = dev ? reinterpret_cast<T*>(z) : b.zp;
+    // A caller's z may overlap its rhs (z == rhs, or views of one buffer). Three launches read all of
+    // rhs before they write z; the one-launch forms do not: the CTAs of the pixel-domain form read
+    // rhs up to ZL_HALO pixels into tiles whose z other CTAs may have written by then, and the
+    // cluster and ticket forms finish some classes before they read others (z == rhs keeps the
+    // classes apart, a shifted view does not). Those solve into the handle's scratch.
+    const uintptr_t r0 = reinterpret_cast<uintptr_t>(rhs), z0 = reinterpret_cast<uintptr_t>(z);
+    const bool overlap = r0 < z0 + nK * sizeof(T) && z0 < r0 + nK * sizeof(T);
+    const bool staged = !dev || (overlap && (zl_now() || ((pl.zf_cs || pl.zs) && r0 != z0)));
+    T* out = staged ? b.zp : reinterpret_cast<T*>(z);
     if ((rc = z_update(src, out))) return rc;
-    if (!dev && (rc = copy_out(z, b.zp, nK, 0))) return rc;
+    if (staged && (rc = copy_out(z, b.zp, nK, dev))) return rc;
     if (pl.zs) {  // the one-launch form waits between its passes (bounded)
       int errflag = 0;
       SGS_CUDA(cudaMemcpyAsync(&errflag, b.err, sizeof(int), cudaMemcpyDeviceToHost, st));
