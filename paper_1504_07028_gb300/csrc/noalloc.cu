@@ -149,8 +149,13 @@ extern "C" int segsalsa_str_linear_solve_static(const float* rhs, float* z, int3
   const size_t col_smem = (size_t)H * CB * sizeof(float2);
   if (col_smem > 200 * 1024) return SEGSALSA_ERR_OOM;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if (c_omega <= ZL_MAX_C) {
-    // the pixel-domain form needs no scratch and no tables
+  // the pixel-domain form needs no scratch and no tables, but its CTAs read rhs in tiles whose z
+  // others may have written by then: overlapping buffers (outside the contract) take the
+  // transforms, which have read all of rhs before they write z
+  const uintptr_t r0 = reinterpret_cast<uintptr_t>(rhs), z0 = reinterpret_cast<uintptr_t>(z);
+  const size_t nb = (size_t)H * W * K * sizeof(float);
+  const bool overlap = r0 < z0 + nb && z0 < r0 + nb;
+  if (c_omega <= ZL_MAX_C && !overlap) {
     ZlArgs za{};
     za.H = H; za.W = W; za.K = K; za.src = rhs; za.z = z;
     za.q = zl_coef(c_omega);

@@ -47,3 +47,22 @@ def test_overlapping_buffers(B, H, W, K, prec, zfuse, wscale):
     s.linear_solve(host, host)
     assert np.array_equal(host, ref.cpu().numpy())
     s.close()
+
+
+@pytest.mark.parametrize("H,W,K", [(145, 145, 16), (300, 313, 16), (64, 96, 5)])
+def test_static_overlapping_buffers(B, H, W, K):
+    """The handle-free call on overlapping buffers: the transforms, for any weights. Tolerance: that of
+    the FP32 transforms against 64 bits in the parity tests."""
+    import torch
+    n, half = H * W * K, (H // 2) * W * K
+    rhs_np = synth.random_field((K, H, W), seed=H + 3 * W).astype(np.float32)
+    ref = khw_to_hwk(O.linear_solve(rhs_np.astype(np.float64), O.gaussian_weights(1, 0.5), 1))
+    rhs = torch.from_numpy(khw_to_hwk(rhs_np)).cuda()
+    for at_r, at_z in ((0, 0), (half, 0), (0, half)):
+        buf = torch.zeros(n + half, device="cuda")
+        buf[at_r:at_r + n] = rhs.flatten()
+        torch.cuda.synchronize()
+        z = buf[at_z:at_z + n].view(H, W, K)
+        assert B.segsalsa_str_linear_solve_static(buf[at_r:at_r + n].view(H, W, K), z) == B.SEGSALSA_OK
+        torch.cuda.synchronize()
+        assert np.abs(z.cpu().numpy() - ref).max() <= 2e-5 * np.abs(ref).max()
