@@ -23,6 +23,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "giveup.h"
 
 namespace sgs {
 
@@ -313,7 +314,7 @@ __global__ void __launch_bounds__(NT, sweep_min_blocks<T, M, DIAG, KEQ, NT>()) k
 
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* mbar = reinterpret_cast<uint64_t*>(smem_raw);  // 2 stage barriers
-  volatile int* gave_up = reinterpret_cast<int*>(smem_raw + 32);
+  const GiveUp gave_up{reinterpret_cast<int*>(smem_raw + 32)};
   const int K = KEQ ? G : a.K;
   const bool cin = !SIMP && a.cin;      // the simplex sweep always reads the full form
   const int dls = cin ? K + 2 : 3 * K;
@@ -350,7 +351,7 @@ __global__ void __launch_bounds__(NT, sweep_min_blocks<T, M, DIAG, KEQ, NT>()) k
     mbar_init(&mbar[0], 1);
     mbar_init(&mbar[1], 1);
     mbar_fence_init();
-    *gave_up = 0;
+    gave_up.clear();
   }
   for (int j = threadIdx.x; j < L; j += NT) om[j] = a.omega[j];
   for (int j = threadIdx.x; j < SB * SBUF; j += NT) slots[j] = T(0);
@@ -430,7 +431,7 @@ __global__ void __launch_bounds__(NT, sweep_min_blocks<T, M, DIAG, KEQ, NT>()) k
   for (int r = 0; r < TH; ++r) {
     const int sidx = r & 1;
     if constexpr (SB == 1) __syncthreads();       // the slots' owners are done with them
-    if (!mbar_wait_bounded(&mbar[sidx], (uint32_t)((r >> 1) & 1), a.budget)) *gave_up = 1;
+    if (!mbar_wait_bounded(&mbar[sidx], (uint32_t)((r >> 1) & 1), a.budget)) gave_up.raise(r);
     const size_t pix0 = (size_t)(y0 + r) * a.W + x0;  // the row's first pixel
     const uint32_t pl = (uint32_t)pix0;               // (its low bits suffice for the offsets)
     unsigned char* st = stage0 + sidx * stb;
@@ -579,7 +580,7 @@ __global__ void __launch_bounds__(NT, sweep_min_blocks<T, M, DIAG, KEQ, NT>()) k
     T* sl = slots + (SB == 2 ? sidx * SBUF : 0);
     flush_write<T, G, NT, E, DIAG>(accW[0], accW2[0], colok, c, g, sl, sl + SLOTS);
     __syncthreads();       // slots written; every thread is past its reads of this row's stage
-    if (*gave_up) {        // uniform: written before the barrier
+    if (gave_up.raised(r)) {   // uniform (giveup.h)
       // a copy never completed: report, give the copies in flight a bounded chance, and leave
       if (threadIdx.x == 0) {
         atomicExch(a.err, 1);
