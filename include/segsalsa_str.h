@@ -135,8 +135,9 @@ int segsalsa_str_solve_until(segsalsa_str_t* h, int32_t max_iters, double tol_pr
 
 /* Bounded device-side waits. The kernels that wait for their own bulk copies (the sweep and
  * the MLR class model) or for the tensor core give up after `cycles` SM clock cycles (default
- * 2e9, about one second), set the handle's error flag, wait once more with the same limit for
- * their copies in flight, release any tensor memory and return; the call then reports
+ * 2e9, about one second), set the handle's error flag, wait once more with the same limit (but
+ * at least 2^21 cycles, about a millisecond) for their copies in flight, release any tensor
+ * memory and return; the call then reports
  * SEGSALSA_ERR_TIMEOUT and the CUDA context stays usable. This is a host-side control, not part
  * of the method (the paper has no counterpart). With probe = 1 the next launches arm their
  * first bulk-copy barrier with 16 bytes that no copy delivers, so that those waits run out by

@@ -25,4 +25,11 @@ struct GiveUp {
   SGS_HD bool raised(int row) const { return flag[row & 1] != 0; }    // between it and the next one
 };
 
+// Clock cycles that a CTA which gave up waits for its copies (or its tensor-core work) still in flight
+// before it reuses their shared memory or exits: the caller's budget, but at least about a
+// millisecond, hundreds of times what a copy takes. Shared memory of a CTA that has exited may
+// belong to another one by the time a late copy lands.
+constexpr long long DRAIN_CYCLES = 1LL << 21;
+SGS_HD long long drain_cycles(long long budget) { return budget > DRAIN_CYCLES ? budget : DRAIN_CYCLES; }
+
 }  // namespace sgs

@@ -12,6 +12,7 @@
 #include <stdint.h>
 
 #include "common.cuh"
+#include "giveup.h"
 
 namespace sgs {
 
@@ -182,7 +183,7 @@ __global__ void __launch_bounds__(MLR_THREADS) k_mlr(const MlrArgs a) {
     // report, and give the staging copies in flight a second bounded chance to land before
     // the buffers are overwritten below (the tile is then computed from zeros and discarded)
     if (threadIdx.x == 0) atomicExch(a.err, 1);
-    mbar_wait_bounded(lbar, 0, a.budget);
+    mbar_wait_bounded(lbar, 0, drain_cycles(a.budget));
   }
   mlr_pack_row(As, stA, threadIdx.x, staged ? rows : 0, a.d, kc);
   if (threadIdx.x < a.npad) mlr_pack_row(Bs, stB, threadIdx.x, staged ? a.K : 0, a.d, kc);
@@ -210,7 +211,7 @@ __global__ void __launch_bounds__(MLR_THREADS) k_mlr(const MlrArgs a) {
     // tensor memory before it exits, so it is freed below either way; the error flag marks
     // the launch's output as invalid (the call returns SEGSALSA_ERR_TIMEOUT and keeps p)
     if (threadIdx.x == 0) atomicExch(a.err, 1);
-    mbar_wait_bounded(bar, 0, a.budget);
+    mbar_wait_bounded(bar, 0, drain_cycles(a.budget));
   } else {
     // epilogue: thread (warp w, lane l) holds the logits of tile row 32w + l
     float lg[32];

@@ -584,8 +584,9 @@ __global__ void __launch_bounds__(NT, sweep_min_blocks<T, M, DIAG, KEQ, NT>()) k
       // a copy never completed: report, give the copies in flight a bounded chance, and leave
       if (threadIdx.x == 0) {
         atomicExch(a.err, 1);
-        mbar_wait_bounded(&mbar[sidx], (uint32_t)((r >> 1) & 1), a.budget);
-        if (r + 1 < TH) mbar_wait_bounded(&mbar[sidx ^ 1], (uint32_t)(((r + 1) >> 1) & 1), a.budget);
+        mbar_wait_bounded(&mbar[sidx], (uint32_t)((r >> 1) & 1), drain_cycles(a.budget));
+        if (r + 1 < TH)
+          mbar_wait_bounded(&mbar[sidx ^ 1], (uint32_t)(((r + 1) >> 1) & 1), drain_cycles(a.budget));
       }
       return;
     }

@@ -1,6 +1,7 @@
-"""The sweep's exit after an exhausted wait (csrc/giveup.h, compiled for the host): in every
-interleaving of a few threads and rows, with one barrier a row, whichever threads give up in
-whichever rows, all threads leave after the same row."""
+"""The exit after an exhausted wait (csrc/giveup.h, compiled for the host): in every interleaving of
+a few threads and rows, with one barrier a row, whichever threads give up in whichever rows, all
+threads of a sweep CTA leave after the same row; and the wait for copies in flight is a
+millisecond at the clock of the GPU (2.07 GHz) however short the budget."""
 import os
 import shutil
 import subprocess
@@ -62,6 +63,8 @@ static void walk(State s) {
     for (int i = 1; i < NT; ++i) parted |= s.t[i].left != s.t[0].left;
 }
 int main() {
+  for (long long b : {1LL, 200000LL, 2000000000LL})
+    if (sgs::drain_cycles(b) < b || sgs::drain_cycles(b) < 2070000LL) { std::printf("drain %lld\n", b); return 1; }
   for (quits = 0; quits < 1u << (NT * ROWS); ++quits) {
     State s{};
     for (auto& x : s.t) x.left = -1;
