@@ -26,6 +26,7 @@
 #include "zfused.cuh"
 #include "zlocal.cuh"
 #include "launch.h"
+#include "tune_key.h"
 #include "mlr.cuh"
 #include "adjoint.cuh"
 #include "wide.cuh"
@@ -1753,24 +1754,20 @@ struct segsalsa_str {
 // lanes run concurrently; replaying the graph costs one launch per chunk.
 namespace sgs {
 
-struct TuneKey {
-  int precision, M, K, size_class;
-  bool operator<(const TuneKey& o) const {
-    return std::tie(precision, M, K, size_class) < std::tie(o.precision, o.M, o.K, o.size_class);
-  }
-};
 static std::mutex g_tune_mu;
 static std::map<TuneKey, segsalsa_str_tiling> g_tune_cache;
 static thread_local std::string g_batch_error;
 
-static int size_class_of(int H, int W) {
-  const long long n = (long long)H * W;
-  int l = 0;
-  while ((2LL << l) <= n) ++l;  // l = floor(log2 n)
-  return l / 2;
+// w: the weights the image was created with (NULL: the Gaussian ones).
+static bool pixel_weights(const segsalsa_str_params& p, const double* w) {
+  segsalsa_str_params q = p;
+  q.weights = w;
+  double c = 0.0;
+  for (double v : make_weights(&q)) c += v * v;
+  return p.precision == SEGSALSA_FP32 && c <= ZL_MAX_C;
 }
-static TuneKey tune_key(const segsalsa_str_params& p) {
-  return TuneKey{p.precision, p.M, p.K, size_class_of(p.H, p.W)};
+static TuneKey tune_key(const segsalsa_str_params& p, const double* w) {
+  return make_tune_key(p.precision, p.M, p.K, p.H, p.W, pixel_weights(p, w));
 }
 static bool same_tiling(const segsalsa_str_tiling& a, const segsalsa_str_tiling& b) {
   return a.tile_rows == b.tile_rows && a.row_pairs == b.row_pairs && a.col_block == b.col_block &&
@@ -1802,6 +1799,7 @@ struct segsalsa_str_batch {
   int* err_host = nullptr;                   // pinned, one flag per image
 
   int fail(int code, const std::string& m) { err = m; return code; }
+  const double* weights_of(int i) const { return weights[i].empty() ? nullptr : weights[i].data(); }
 #define SGB_CUDA(call)                                                                       \
   do {                                                                                       \
     cudaError_t e_ = (call);                                                                 \
@@ -1837,7 +1835,7 @@ struct segsalsa_str_batch {
   int make_image(int i, const segsalsa_str_tiling* t, std::unique_ptr<sgs::SolverBase>& out) {
     std::string msg;
     segsalsa_str_params pr = params[i];
-    pr.weights = weights[i].empty() ? nullptr : weights[i].data();
+    pr.weights = weights_of(i);
     pr.stream = nullptr;
     const int rc = sgs::create_any(&pr, nullptr, 0, out, msg, t);
     if (rc) return fail(rc, "image " + std::to_string(i) + ": " + msg);
@@ -1862,7 +1860,7 @@ struct segsalsa_str_batch {
         req[i] = tl[i];
       } else {
         std::lock_guard<std::mutex> g(sgs::g_tune_mu);
-        auto it = sgs::g_tune_cache.find(sgs::tune_key(pr[i]));
+        auto it = sgs::g_tune_cache.find(sgs::tune_key(pr[i], pr[i].weights));
         req[i] = it != sgs::g_tune_cache.end() ? it->second : segsalsa_str_tiling{0, 0, 0, 0, 0};
       }
     }
@@ -2092,7 +2090,7 @@ struct segsalsa_str_batch {
     }
     // then the tiling of each class, largest total work first
     std::map<sgs::TuneKey, std::vector<int>> groups;
-    for (int i = 0; i < n; ++i) groups[sgs::tune_key(params[i])].push_back(i);
+    for (int i = 0; i < n; ++i) groups[sgs::tune_key(params[i], weights_of(i))].push_back(i);
     std::vector<std::pair<double, sgs::TuneKey>> order;
     for (auto& kv : groups) {
       double w = 0;
@@ -2115,18 +2113,13 @@ struct segsalsa_str_batch {
         key.clear();
         for (int i : mem) {
           segsalsa_str_params pr = params[i];
-          pr.weights = weights[i].empty() ? nullptr : weights[i].data();
+          pr.weights = weights_of(i);
           sgs::Plan pl;
           std::string msg;
           const int rc = pr.precision == SEGSALSA_FP32 ? sgs::make_plan<float>(&pr, pl, msg, &t)
                                                        : sgs::make_plan<double>(&pr, pl, msg, &t);
           if (rc) return false;
-          key.push_back(pl.THmax); key.push_back(pl.zl);
-          if (pl.zl) continue;                  // no row or column pass to tile
-          key.push_back(pl.QB); key.push_back(pl.CB);
-          key.push_back(pl.row.threads); key.push_back(pl.NSEG); key.push_back(pl.zf_cs);
-          key.push_back(pl.rp);
-          key.push_back(pl.p2);
+          sgs::append_tiling_key(key, pl, sgs::pixel_weights(pr, pr.weights));
         }
         return true;
       };
