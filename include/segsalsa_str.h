@@ -242,20 +242,23 @@ int segsalsa_str_get_probs(segsalsa_str_t* h, void* p, int32_t layout, int32_t o
  * with periodic boundaries, which is the z-update operator (3 I + J^T J) of a handle whose shift
  * weights have sum_j omega_j^2 = c_omega (1 for the default normalised Gaussian weights).
  *  - rhs, z: FP32 device memory, pixel-major (H, W, K), owned by the caller; z may not alias rhs.
- *  - Scratch: one file-scope device array (16 MiB spectrum + 512 KiB tables) that every GPU
- *    loading the library holds until exit. Limits: H*(W/2+1)*K <= 2097152, W <= 8192 when W has
- *    no prime factor above 7 and W <= 4096 otherwise, H <= 3200, 2 <= H, W, 1 <= K <= 32.
- *    Sizes beyond them return SEGSALSA_ERR_OOM; other bad arguments SEGSALSA_ERR_ARG.
- *  - No cudaMalloc / cudaFree or other device allocation happens in any call. Every call looks
- *    up the array's device address in the current context (cudaGetSymbolAddress, which
- *    allocates nothing). The first call on a device, and the first call after H, W or c_omega
- *    change or after the device was reset (a new context), builds the tables with two small
- *    kernels on `stream` before the solve; make the first call before any stream capture.
+ *  - Limits, whatever c_omega: H*(W/2+1)*K <= 2097152, W <= 8192 when W has no prime factor
+ *    above 7 and W <= 4096 otherwise, H <= 3200, 2 <= H, W, 1 <= K <= 32. Sizes beyond them
+ *    return SEGSALSA_ERR_OOM; other bad arguments SEGSALSA_ERR_ARG. No cudaMalloc / cudaFree or
+ *    other device allocation happens in any call.
+ *  - c_omega <= 1.0005 (normalised weights): one kernel in the pixel domain, without scratch.
+ *  - Larger c_omega: row transforms and column solves, with scratch in one file-scope device array
+ *    (16 MiB spectrum + 512 KiB tables) that every GPU loading the library holds until exit.
+ *    Such a call looks up the array's device address in the current context
+ *    (cudaGetSymbolAddress, which allocates nothing). The first one on a device, and the first
+ *    after H, W or c_omega change or after the device was reset (a new context), builds the
+ *    tables with two small kernels on `stream` before the solve; make it before any stream
+ *    capture. Nothing in the array needs to start at zero, because each call writes every
+ *    spectrum entry it reads.
  *  - Runs asynchronously on `stream` (cudaStream_t, NULL = legacy default stream). Calls on one
- *    stream may follow each other with any geometries and no synchronisation in between. Every
- *    call shares the one array, so calls that overlap on the GPU (different streams, other
- *    threads) race; nothing in it needs to start at zero, because each call writes every
- *    spectrum entry it reads. The host-side bookkeeping is locked, but concurrent calls are
+ *    stream may follow each other with any geometries and no synchronisation in between. Calls
+ *    with larger c_omega share the one array, so those that overlap on the GPU (different
+ *    streams, other threads) race; the host-side bookkeeping is locked, but concurrent calls are
  *    still unsupported for that reason. No message is stored: the status code is the error
  *    report. */
 int segsalsa_str_linear_solve_static(const float* rhs, float* z, int32_t H, int32_t W, int32_t K,
@@ -310,11 +313,11 @@ int segsalsa_str_traffic_model(const segsalsa_str_t* h, double* sweep_bytes,
  *                 more than 512 threads; one-unit row form only; measured slower than the
  *                 three launches chained by programmatic dependent launch: 145x145, K = 16,
  *                 36.3 vs 30.8 us per iteration); 0 = the library's choice: in FP32, with
-                 row_pipe = 0 and weights whose squared sum is at most 1 (the Gaussian ones),
-                 one launch in the pixel domain (no transforms: the other fields but tile_rows
-                 are then unused), else three launches. get_tiling reports zfuse = 1 and
-                 row_pipe = 0 for a handle that leaves this choice to the library, and a
-                 complete tiling with those two values leaves it too.
+ *                 row_pipe = 0 and weights whose squares sum to at most 1.0005 (the Gaussian
+ *                 ones: 1), one launch in the pixel domain (no transforms: the other fields
+ *                 but tile_rows are then unused), else three launches. get_tiling reports
+ *                 zfuse = 1 and row_pipe = 0 for a handle that leaves this choice to the
+ *                 library, and a complete tiling with those two values leaves it too.
  *                 A fused request that the band or the device cannot hold runs three
  *                 launches (get_tiling reports 1).
  *   row_pipe    : form of the two row-transform passes: 1 = one CTA per (row, class block);
@@ -352,8 +355,9 @@ typedef struct segsalsa_str_batch segsalsa_str_batch_t; /* opaque; owned by the 
  * params[i].stream must be NULL (each image gets a library stream; the graphs run on
  * `stream`, a borrowed cudaStream_t, or a library stream when NULL). tiling (nullable) holds
  * n_images entries; when NULL each image takes the tiling that segsalsa_str_batch_autotune
- * chose for its class (precision, M, K, size class floor(log2(H W) / 2)) earlier in this
- * process, else the defaults. Device memory: the sum of the images' workspace_bytes. */
+ * chose for its class (precision, M, K, size class floor(log2(H W) / 2), and whether the weights
+ * given here allow the pixel-domain z-update) earlier in this process, else the defaults. Device
+ * memory: the sum of the images' workspace_bytes. */
 int segsalsa_str_batch_create(int32_t n_images, const segsalsa_str_params* params,
                               const segsalsa_str_tiling* tiling, void* stream,
                               segsalsa_str_batch_t** out);
@@ -373,7 +377,7 @@ int segsalsa_str_batch_solve(segsalsa_str_batch_t* b, int32_t iters);
  * class, largest total work first, times `trial_iters` >= 1 batch iterations for every
  * candidate tiling of that class while the other classes keep their current tiling, keeping
  * the fastest (candidates: tile_rows 4..32, then row_pairs, col_block, row_threads,
- * col_rows and row_pipe in turn). The lane count
+ * col_rows and row_pipe in turn; those that leave what runs unchanged are skipped). The lane count
  * is tuned first the same way (4, 8, 16, 32, n_images). The choice is
  * stored per class in a process-wide cache (used by later batch_create calls with tiling ==
  * NULL) and written to chosen[i] (nullable, n_images entries). The images are rebuilt with

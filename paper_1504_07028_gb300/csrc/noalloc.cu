@@ -4,12 +4,14 @@
 // inside a region that must not call cudaMalloc (it synchronises the device and can fail
 // under a fixed memory budget), under an external allocator that owns all device memory, or
 // from a plug-in that has no handle and cannot keep one. Such callers pass their own rhs and
-// z buffers; the scratch this operation needs (the row spectrum and the transform tables)
-// lives in one file-scope device array of fixed size that every GPU loading the library
-// holds until the process exits.
+// z buffers.
 //
-// The kernels are the library's own row-DFT and column-solve passes; only the memory they
-// work in differs. Host code never dereferences g_static_scratch: the array's name on the
+// For c_omega up to ZL_MAX_C (the normalised weights among them) the pixel-domain kernels of zlocal.cu
+// solve the system in one launch with no scratch and no tables. Larger c_omega runs the
+// library's row-DFT and column-solve passes, whose scratch (the row spectrum and the transform
+// tables) lives in one file-scope device array of fixed size that every GPU loading the library
+// holds until the process exits; the rest of this comment is about those. The size limits are the
+// array's and hold for every c_omega. Host code never dereferences g_static_scratch: the array's name on the
 // host is a stand-in, not a device address, so its device address is looked up with
 // cudaGetSymbolAddress on every call (with the caller's device current; the lookup allocates
 // nothing). The transform tables kept in the array are rebuilt whenever the geometry, the

@@ -9,8 +9,9 @@
 //   d_j <- u_j - v_j  (= d_j - (G z - u_j), eq. 14)
 //   rhs = (u1 + d1) + J^T (u2 + d2) + (u3 + d3) + (u4 + d4)              (G^T (u + d), eq. 12)
 //
-// Work mapping. A CTA owns a tile of pixels (balanced tiling of the image) and 256 threads:
-// NC = 256/G columns x G lanes. The G lanes of a column hold the classes of one pixel (class
+// Work mapping. A CTA owns a tile of pixels (balanced tiling of the image) and NT = 256 threads,
+// or 64 where the image has fewer than 152 tiles of 256: NC <= NT / G columns x G lanes. The G
+// lanes of a column hold the classes of one pixel (class
 // k = lane), so the 2x2 Gram matrix [Jz]_i^T [Jz]_i of eq. (5) is a G-lane shuffle sum and
 // each lane keeps its 2L Jacobian entries in registers. Each column walks down the tile rows.
 // The Jacobian stencil reads z from a shared-memory copy of the tile plus its halo
@@ -18,8 +19,9 @@
 // (2M+2)^2 neighbours i + s_j (+ e_h / e_v). Each thread keeps those sums for the rows it can
 // still touch in a (2M+2)x(2M+2) register window; every row step, the finished top window row
 // goes through exclusive shared-memory slots, is summed in a fixed order by the owner of each
-// column and stored as one row of the tile's partials P (tile plus halo). The row-FFT pass
-// adds the overlapping tiles when it reads rhs (no atomics anywhere: deterministic).
+// column and stored as one row of the tile's partials P (tile plus halo). The z-update (the
+// pixel-domain kernels of zlocal.cu, or the row transforms of fft.cuh) adds the overlapping tiles
+// when it reads rhs (no atomics anywhere: deterministic).
 #pragma once
 
 #include "common.cuh"
@@ -30,7 +32,7 @@ namespace sgs {
 template <typename T>
 struct SweepArgs {
   int H, W, K;
-  int NC;                // columns per tile (<= 256 / G)
+  int NC;                // columns per tile (<= threads / G)
   int ntx, nty;          // tile grid
   int EHmax, EWmax;      // extents of the P tile slots (tile + halo), in pixels
   const T* z;            // [n][K]

@@ -1,6 +1,6 @@
 // z-update (12) of SegSALSA-STR in the pixel domain, one launch: z = (3 I + J^T J)^{-1} rhs.
 //
-// With weights normalised as the method's Gaussian ones (c = sum_j omega_j^2 <= 1) the 5-point
+// With weights normalised as the method's Gaussian ones (c = sum_j omega_j^2 = 1, or less) the 5-point
 // operator A = d - c (S_x + S_x^{-1} + S_y + S_y^{-1}), d = 3 + 4c, is so well conditioned
 // (eigenvalues in [3, 3 + 8c]) that its inverse is local: it decays by 0.209 or less per
 // pixel, and the Chebyshev semi-iteration (Golub and Varga) on the Jacobi splitting
@@ -12,9 +12,12 @@
 // on random fields: 5.1e-8 relative, where the row transforms and column recursions of fft.cuh,
 // which every other case takes (FP64, larger weights), leave 1.8e-7.
 //
-// A strip is computed from its pixels and a halo of ZL_HALO: beyond it the right-hand side is
-// taken as 0, an error of at most 0.209^12 = 7e-9 of it at the strip's edge. Nothing depends on
-// the image's size: no transform length, no period (halo pixels wrap), any class count.
+// A strip is computed from its pixels and a halo of ZL_HALO. What lies beyond counts as 0, except at
+// the first and last column of the streaming form, whose missing neighbour is replaced by a value of
+// the same lane's four columns (a shuffle past the end of the warp returns it): either way a neighbour off
+// by at most twice the field's largest value, of which 0.209^12 = 7e-9 reaches the wanted pixels.
+// Nothing depends on the image's size: no transform length, no period (halo pixels wrap), any
+// class count.
 #pragma once
 
 #include <algorithm>
@@ -89,7 +92,9 @@ struct ZlArgs {
 // Work split of the smaller modelled time (us on one GB300; the constants fit event times of both
 // forms over 64 x 64, K = 4 to 2048 x 2048, K = 16). Streaming: two CTAs an SM, 0.45 us a row with
 // both at work and 0.38 us alone, a segment of h rows taking h + 28 of them. Block form: one CTA
-// an SM, 3.5 us and 0.0065 us a thread (more where only one class of a quad is loaded).
+// an SM, 3.5 us and 0.0065 us a thread (more where only one class of a quad is loaded). The model has
+// one image on an idle GPU in mind; the images of a batch, which share it, take the same split
+// all the same, because each has to match its own handle bit for bit and results depend on the split.
 inline ZlPlan zl_plan(int H, int W, int K) {
   const int sms = 152, edge = 2 * ZL_HALO, useful = ZL_WIDTH - edge;
   ZlPlan p{(W + useful - 1) / useful, 1, 0, 0, 0, 128};
